@@ -121,6 +121,7 @@ __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, 
                               int n_chunks, int per_chunk, const float *__restrict__ part_m,
                               const float *__restrict__ part_z, float *__restrict__ rowb, long units)
 {
+    wait_prior_grid();  // the partials come from pass 1
     long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= units * R) return;
     long u = i / R;
@@ -129,45 +130,21 @@ __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, 
     if (L < w || L > L_cap || mask.skip(u, L, w, L_cap)) return;
     int used = ((L + kScoreChunk - 1) / kScoreChunk) * per_chunk;
     float m = -INFINITY, z = 0.f;
-    for (int c = 0; c < used; ++c) {
-        size_t o = ((size_t)u * n_chunks * per_chunk + c) * R + r;
-        lse_merge(m, z, part_m[o], part_z[o]);
+    const size_t o0 = (size_t)u * n_chunks * per_chunk * R + r;
+    constexpr int U = 8;  // partials in flight
+    for (int c0 = 0; c0 < used; c0 += U) {
+        float pm[U], pz[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const bool in = c0 + k < used;
+            const size_t o = o0 + (size_t)(c0 + k) * R;
+            pm[k] = in ? part_m[o] : -INFINITY;
+            pz[k] = in ? part_z[o] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) lse_merge(m, z, pm[k], pz[k]);
     }
     rowb[i] = m + log2f(z);
-}
-
-// The units a masked call scores, in ascending order (one CTA; a ballot scan per
-// blockDim.x units), and their count.
-__device__ __forceinline__ void unit_list_block(const int32_t *__restrict__ lens, ScoreMask mask, int w, int L_cap,
-                                                int units, int32_t *__restrict__ ulist, int32_t *__restrict__ ucount)
-{
-    __shared__ int warp_n[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int base = 0;
-    for (int u0 = 0; u0 < units; u0 += blockDim.x) {
-        const int u = u0 + threadIdx.x;
-        const bool take = u < units && !mask.skip(u, lens[u], w, L_cap);
-        const unsigned bal = __ballot_sync(0xffffffffu, take);
-        if (lane == 0) warp_n[wid] = __popc(bal);
-        __syncthreads();
-        int off = base, tot = 0;
-        for (int k = 0; k < nw; ++k) {
-            off += k < wid ? warp_n[k] : 0;
-            tot += warp_n[k];
-        }
-        if (take) ulist[off + __popc(bal & ((1u << lane) - 1u))] = u;
-        base += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *ucount = base;
-}
-
-__global__ void __launch_bounds__(1024) score_unit_list(const int32_t *__restrict__ lens, ScoreMask mask, int w,
-                                                        int L_cap, int units, int32_t *__restrict__ ulist,
-                                                        int32_t *__restrict__ ucount)
-{
-    wait_prior_grid();
-    unit_list_block(lens, mask, w, L_cap, units, ulist, ucount);
 }
 
 // Row normalisers from log-sum-exps the decode already produced (Eq. 2 with one pass over
@@ -314,57 +291,147 @@ __global__ void __launch_bounds__(128) score_colsum_simt(
     }
 }
 
-// Max-pool over the clipped window [j - pool/2, j + pool/2] within [0, L-w).
-// score_pool over the units of a masked call's list only: CTAs (blockIdx.x: a 256-key
-// chunk) walk the list, so the units left out cost no CTAs.
-__global__ void score_pool_list(const float *__restrict__ raw, const int32_t *__restrict__ lens,
-                                const int32_t *__restrict__ ulist, const int32_t *__restrict__ ucount, int w,
-                                int L_cap, int pool, float *__restrict__ scores)
+// Max-pool over the clipped window [j - pool/2, j + pool/2] within [0, L-w).  A CTA pools
+// kPoolTile scores of a unit from a shared-memory copy of them and their halo; scores outside the
+// range are NaN there, which fmaxf passes over, so that no window needs clipping.  What bounds it
+// is latency (length, scores, barrier, results), so a thread keeps 16 scores in flight: 7B-class
+// cache, 14.2 M scores, took 55 us with one load per window entry.  Windows wider than the halo read global memory.
+constexpr int kPoolTile = 4096, kPoolHalo = 64, kPoolThreads = 256;
+
+__device__ __forceinline__ void pool_tile(const float *__restrict__ rp, int j0, int nc, int half,
+                                          float *__restrict__ out, bool vec, float *sm)
 {
+    constexpr int Q = kPoolTile / kPoolThreads / 4;  // groups of four consecutive scores per thread
+    const int n = min(kPoolTile, nc - j0);
+    if (half > kPoolHalo) {
+        for (int t = threadIdx.x; t < n; t += kPoolThreads) {
+            const int j = j0 + t, lo = max(0, j - half), hi = min(nc - 1, j + half);
+            float m = rp[lo];
+            for (int i = lo + 1; i <= hi; ++i) m = fmaxf(m, rp[i]);
+            out[j] = m;
+        }
+        return;
+    }
+    const float none = __int_as_float(0x7fc00000);
+    float *c = sm + kPoolHalo;  // c[t] = score j0 + t
+    if (vec) {                  // rows of whole, aligned groups of four (the group at nc stays inside the row)
+        float4 v[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int t = 4 * (threadIdx.x + q * kPoolThreads);
+            v[q] = t < n ? __ldcg(reinterpret_cast<const float4 *>(rp + j0 + t)) : make_float4(none, none, none, none);
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int t = 4 * (threadIdx.x + q * kPoolThreads);
+            if (t + 1 >= n) v[q].y = none;
+            if (t + 2 >= n) v[q].z = none;
+            if (t + 3 >= n) v[q].w = none;
+            *reinterpret_cast<float4 *>(c + t) = v[q];
+        }
+    } else {
+        float v[4 * Q];
+#pragma unroll
+        for (int q = 0; q < 4 * Q; ++q) {
+            const int t = threadIdx.x + q * kPoolThreads;
+            v[q] = t < n ? __ldcg(rp + j0 + t) : none;
+        }
+#pragma unroll
+        for (int q = 0; q < 4 * Q; ++q) c[threadIdx.x + q * kPoolThreads] = v[q];
+    }
+    if (threadIdx.x < 2 * kPoolHalo) {
+        const int t = threadIdx.x < kPoolHalo ? (int)threadIdx.x - kPoolHalo : kPoolTile + (int)threadIdx.x - kPoolHalo;
+        const int j = j0 + t;
+        c[t] = j >= 0 && j < nc && t >= -half && t < kPoolTile + half ? __ldcg(rp + j) : none;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const int t = 4 * (threadIdx.x + q * kPoolThreads);
+        if (t >= n) break;
+        float m[4];
+        if (half <= 4) {
+            float x[12];  // scores t - 4 .. t + 7
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 f = *reinterpret_cast<const float4 *>(c + t - 4 + 4 * i);
+                x[4 * i] = f.x;
+                x[4 * i + 1] = f.y;
+                x[4 * i + 2] = f.z;
+                x[4 * i + 3] = f.w;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                m[k] = x[4 + k];
+#pragma unroll
+                for (int o = 1; o <= 4; ++o)
+                    if (o <= half) m[k] = fmaxf(m[k], fmaxf(x[4 + k - o], x[4 + k + o]));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m[k] = none;
+            for (int i = -half; i < half + 4; ++i) {
+                const float x = c[t + i];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (i >= k - half && i <= k + half) m[k] = fmaxf(m[k], x);
+            }
+        }
+        if (vec && t + 4 <= n) {
+            *reinterpret_cast<float4 *>(out + j0 + t) = make_float4(m[0], m[1], m[2], m[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (t + k < n) out[j0 + t + k] = m[k];
+        }
+    }
+    __syncthreads();
+}
+
+// Whether a unit's rows of raw and scores are whole, aligned groups of four.
+__device__ __forceinline__ bool pool_vec(const float *raw, const float *scores, int L_cap)
+{
+    return (L_cap & 3) == 0 && ((reinterpret_cast<uintptr_t>(raw) | reinterpret_cast<uintptr_t>(scores)) & 15u) == 0;
+}
+
+// The pool over the units of a masked call's list only: CTAs (blockIdx.x: a tile of scores)
+// walk the list, so the units left out cost no CTAs.
+__global__ void __launch_bounds__(kPoolThreads) score_pool_list(const float *__restrict__ raw, const int32_t *__restrict__ lens,
+                                                       const int32_t *__restrict__ ulist,
+                                                       const int32_t *__restrict__ ucount, int w, int L_cap, int pool,
+                                                       float *__restrict__ scores)
+{
+    __shared__ __align__(16) float sm[kPoolTile + 2 * kPoolHalo];
     wait_prior_grid();  // the raw scores and the list come from the previous kernels
     const int n = *ucount;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int half = pool / 2;
     for (int k = blockIdx.y; k < n; k += gridDim.y) {
         const long u = ulist[k];
-        const int L = lens[u];
-        if (L < w || L > L_cap) continue;
-        const int nc = L - w;
-        if (j >= nc) continue;
-        const int lo = max(0, j - half), hi = min(nc - 1, j + half);
-        const float *rp = raw + u * L_cap;
-        float m = rp[lo];
-        for (int i = lo + 1; i <= hi; ++i) m = fmaxf(m, rp[i]);
-        scores[u * L_cap + j] = m;
+        const int L = lens[u], j0 = blockIdx.x * kPoolTile;
+        if (L < w || L > L_cap || j0 >= L - w) continue;
+        pool_tile(raw + u * L_cap, j0, L - w, pool / 2, scores + u * L_cap, pool_vec(raw, scores, L_cap), sm);
     }
 }
 
-__global__ void score_pool(const float *__restrict__ raw, const int32_t *__restrict__ lens, ScoreMask mask, int w,
-                           int L_cap, int pool, float *__restrict__ scores)
+__global__ void __launch_bounds__(kPoolThreads) score_pool(const float *__restrict__ raw, const int32_t *__restrict__ lens,
+                                                  ScoreMask mask, int w, int L_cap, int pool,
+                                                  float *__restrict__ scores)
 {
+    __shared__ __align__(16) float sm[kPoolTile + 2 * kPoolHalo];
     wait_prior_grid();  // the raw scores come from the previous kernel
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
     const long u = blockIdx.y;
-    const int L = lens[u];
-    if (L < w || L > L_cap || mask.skip(u, L, w, L_cap)) return;
-    const int nc = L - w;
-    if (j >= nc) return;
-    const int half = pool / 2;
-    const int lo = max(0, j - half), hi = min(nc - 1, j + half);
-    const float *rp = raw + u * L_cap;
-    float m = rp[lo];
-    for (int i = lo + 1; i <= hi; ++i) m = fmaxf(m, rp[i]);
-    scores[u * L_cap + j] = m;
+    const int L = lens[u], j0 = blockIdx.x * kPoolTile;
+    if (L < w || L > L_cap || mask.skip(u, L, w, L_cap) || j0 >= L - w) return;
+    pool_tile(raw + u * L_cap, j0, L - w, pool / 2, scores + u * L_cap, pool_vec(raw, scores, L_cap), sm);
 }
 
-
-cudaError_t launch_score_tc_pass1(const reco_kv &kv, const void *q_win, const int32_t *lens, bool masked, int w,
-                                  float c2, const ScoreWs &ws, unsigned *err, cudaStream_t s, bool *used);
+cudaError_t launch_score_tc_pass1(const reco_kv &kv, const void *q_win, const int32_t *lens, const ScoreMask &mask,
+                                  int w, float c2, const ScoreWs &ws, unsigned *err, cudaStream_t s, bool *used);
 // row_lse (or nullptr: ws.rowb) gives pass 2 its row normalisers: the decode's lse, read
 // where each row's normaliser is loaded.
-cudaError_t launch_score_tc_pass2(const reco_kv &kv, const void *q_win, const int32_t *lens, bool masked, int w,
-                                  float c2, const ScoreWs &ws, const float *row_lse, unsigned *err, cudaStream_t s,
-                                  bool *used);
+// A masked call's pass 2 also lists the units it scored in ws.ulist / ws.ucount.
+cudaError_t launch_score_tc_pass2(const reco_kv &kv, const void *q_win, const int32_t *lens, const ScoreMask &mask,
+                                  int w, float c2, const ScoreWs &ws, const float *row_lse, unsigned *err,
+                                  cudaStream_t s, bool *used);
 bool score_tc_supported(const reco_kv &kv, int w);
 int score_tc_pass1_groups(int R);
 
@@ -421,20 +488,20 @@ static cudaError_t score_simt_any(const reco_kv &kv, const void *q_win, const in
 }
 
 // Max-pooling of the raw scores into `scores`: over the unit list when the call built one
-// (a masked tensor-core call), else one CTA per (unit, 256-key chunk).
+// (a masked tensor-core call), else one CTA per (unit, tile of scores).
 static cudaError_t launch_pool(const reco_kv &kv, const int32_t *lens, ScoreMask mask, bool listed, int w, int pool,
                                float *scores, const ScoreWs &ws, cudaStream_t s)
 {
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
-    const unsigned chunks = (unsigned)((kv.L_cap + 255) / 256);
+    const unsigned chunks = (unsigned)((kv.L_cap + kPoolTile - 1) / kPoolTile);
     if (listed) {
         const long walkers = std::max(1L, 8L * device_sm_count() / (long)chunks);
         const unsigned ys = (unsigned)std::min(units, std::min(walkers, 65535L));
-        cudaError_t e = launch_pdl(score_pool_list, dim3(chunks, ys), dim3(256), 0, s, (const float *)ws.raw, lens,
+        cudaError_t e = launch_pdl(score_pool_list, dim3(chunks, ys), dim3(kPoolThreads), 0, s, (const float *)ws.raw, lens,
                                    (const int32_t *)ws.ulist, (const int32_t *)ws.ucount, w, kv.L_cap, pool, scores);
         if (e != cudaSuccess) return e;
     } else {
-        cudaError_t e = launch_pdl(score_pool, dim3(chunks, (unsigned)units), dim3(256), 0, s, (const float *)ws.raw, lens,
+        cudaError_t e = launch_pdl(score_pool, dim3(chunks, (unsigned)units), dim3(kPoolThreads), 0, s, (const float *)ws.raw, lens,
                                    mask, w, kv.L_cap, pool, scores);
         if (e != cudaSuccess) return e;
     }
@@ -451,22 +518,18 @@ cudaError_t launch_score(const reco_kv &kv, const void *q_win, const int32_t *le
     bool used_tc = false;
     const bool tc = kv.dtype == RECO_BF16 && score_tc_supported(kv, w);
     if (tc) {
-        // tensor-core passes: (unit list) -> pass 1 -> combine -> pass 2
-        if (keep) {
-            e = launch_pdl(score_unit_list, dim3(1), dim3(1024), 0, s, lens, mask, w, kv.L_cap, (int)units, ws.ulist,
-                           ws.ucount);
-            if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
-        }
-        e = launch_score_tc_pass1(kv, q_win, lens, keep != nullptr, w, c2, ws, err, s, &used_tc);
+        // tensor-core passes: pass 1 -> combine -> pass 2
+        e = launch_score_tc_pass1(kv, q_win, lens, mask, w, c2, ws, err, s, &used_tc);
         if (e != cudaSuccess) return e;
         if (used_tc) {
             const int R = (kv.H_q / kv.H_kv) * w;
             const int nch = (kv.L_cap + kScoreChunk - 1) / kScoreChunk;
-            score_combine<<<(unsigned)((units * R + 255) / 256), 256, 0, s>>>(
-                lens, mask, w, kv.L_cap, R, nch, score_tc_pass1_groups(R), ws.part_m, ws.part_z, ws.rowb, units);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            e = launch_pdl(score_combine, dim3((unsigned)((units * R + 255) / 256)), dim3(256), 0, s, lens, mask, w,
+                           kv.L_cap, R, nch, score_tc_pass1_groups(R), (const float *)ws.part_m,
+                           (const float *)ws.part_z, ws.rowb, units);
+            if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
             bool used2 = false;
-            e = launch_score_tc_pass2(kv, q_win, lens, keep != nullptr, w, c2, ws, nullptr, err, s, &used2);
+            e = launch_score_tc_pass2(kv, q_win, lens, mask, w, c2, ws, nullptr, err, s, &used2);
             if (e != cudaSuccess) return e;
             if (!used2) return cudaErrorNotSupported;
         }
@@ -475,7 +538,7 @@ cudaError_t launch_score(const reco_kv &kv, const void *q_win, const int32_t *le
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, true);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, tc && keep, w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used_tc && keep, w, pool, scores, ws, s);
 }
 
 cudaError_t launch_lse_push(const float *lse, long n, float *ring, int slots, long long *slot, unsigned *err,
@@ -539,12 +602,7 @@ cudaError_t launch_score_lse(const reco_kv &kv, const void *q_win, const int32_t
     cudaError_t e;
     bool used = false;
     if (tc) {  // the tensor-core pass reads each row's normaliser from row_lse itself
-        if (keep) {
-            e = launch_pdl(score_unit_list, dim3(1), dim3(1024), 0, s, lens, mask, w, kv.L_cap, (int)units, ws.ulist,
-                           ws.ucount);
-            if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
-        }
-        e = launch_score_tc_pass2(kv, q_win, lens, keep != nullptr, w, c2, ws, row_lse, err, s, &used);
+        e = launch_score_tc_pass2(kv, q_win, lens, mask, w, c2, ws, row_lse, err, s, &used);
         if (e != cudaSuccess) return e;
     }
     if (!used) {  // the SIMT pass takes them from ws.rowb
@@ -554,7 +612,7 @@ cudaError_t launch_score_lse(const reco_kv &kv, const void *q_win, const int32_t
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, false);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, tc && keep, w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used && keep, w, pool, scores, ws, s);
 }
 
 }  // namespace reco

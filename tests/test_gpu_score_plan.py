@@ -1,0 +1,61 @@
+"""The tensor-core scoring's work plan and column ranges, and the pool's tiles, against the oracle:
+window-row counts whose halves end in 8 columns, ranges of more than one plan round, pools that
+cross tiles, exceed the shared-memory halo or meet unaligned rows."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from helpers import assert_scores_close, gpu_score, np32
+from paper_2608_04771_gb300 import reco
+from paper_2608_04771_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_2608_04771_gb300 import build
+    build.build()
+    reco.lib()
+
+
+def _check(wl, lens, pool, units):
+    K, V = W.make_cache(wl, DEV, canary=False)
+    q = W.make_qwin(wl, DEV)
+    got = gpu_score(wl, K, V, q, torch.from_numpy(lens).to(DEV), pool).cpu().numpy()
+    reco.reco_check()
+    G = wl.h_q // wl.h_kv
+    for l, b, h in units:
+        L = int(lens[l, b, h])
+        _, ora = oracle.score_unit(np32(q[l, b, h * G:(h + 1) * G]), np32(K[l, b, h, :L]), wl.w, wl.scale(), pool)
+        assert_scores_close(got[l, b, h, :L - wl.w], ora, f"unit {(l, b, h)}")
+
+
+# window rows G * w: 5 and 16 (one 8-column half), 48 (16 + 8), 112, 130 (144 columns, three regions),
+# 272 (two chains of 144), 384 (three query tiles), 400 and 512 (four)
+@pytest.mark.parametrize("G,w,d", [(1, 5, 64), (1, 16, 128), (3, 16, 128), (7, 16, 64), (13, 10, 128), (17, 16, 128),
+                                   (12, 32, 64), (8, 50, 128), (16, 32, 128)])
+def test_window_row_counts(G, w, d):
+    wl = W.WORKLOADS["7b"].reduced(layers=2, batch=2, h_q=2 * G, h_kv=2, d=d, L=2300, decode_steps=5, w=w)
+    rng = np.random.default_rng(G * 100 + w)
+    lens = rng.integers(w, 2306, (2, 2, 2)).astype(np.int32)
+    lens[0, 0, 0], lens[1, 1, 1] = 2048 + w, w + 1
+    _check(wl, lens, 7, [(0, 0, 0), (0, 1, 1), (1, 0, 0), (1, 1, 1)])
+
+
+def test_more_units_than_one_plan_round():
+    """About 300 units per CTA of one or two tiles each: two rounds of 256 runs."""
+    wl = W.WORKLOADS["7b"].reduced(layers=64, batch=89, h_q=8, h_kv=8, d=64, L=200, decode_steps=0, w=8)
+    rng = np.random.default_rng(3)
+    lens = rng.integers(8, 201, (64, 89, 8)).astype(np.int32)
+    units = [tuple(int(x) for x in np.unravel_index(i, lens.shape)) for i in rng.integers(0, lens.size, 40)]
+    _check(wl, lens, 3, units + [(0, 0, 0), (63, 88, 7)])
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("L,pool", [(4240, 7), (4241, 9), (4240, 21), (4243, 129), (4240, 131), (8300, 1)])
+def test_pool_tiles(dtype, L, pool):
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=1, h_q=4, h_kv=2, d=64, L=L, decode_steps=0, w=16, dtype=dtype)
+    _check(wl, np.array([[[L, 4096 + 17 if L < 8000 else 4111]]], np.int32), pool, [(0, 0, 0), (0, 0, 1)])
