@@ -16,14 +16,27 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "score_plan.cuh"
 
 namespace reco {
+
+bool score_tc_supported(const reco_kv &kv, int w);
+
+// Partials of a window row in the workspace.  Tensor-core shapes: up to two per chunk (a chunk's
+// key tiles are split between two epilogue groups).  Others: one per tile of keys, so that the
+// tiles of a short call spread over the SMs.
+static int score_row_parts(const reco_kv &kv, int w)
+{
+    return score_tc_supported(kv, w) ? 2 * ((kv.L_cap + kScoreChunk - 1) / kScoreChunk) : (kv.L_cap + kTile - 1) / kTile;
+}
+
+// Tiles per partial on plain FMAs (a tensor-core shape gets there only without tensor maps).
+static int simt_part_tiles(const reco_kv &kv, int w) { return score_tc_supported(kv, w) ? kScoreChunk / kTile : 1; }
 
 ScoreWs score_ws_layout(const reco_kv &kv, int w, void *base)
 {
     size_t units = (size_t)kv.n_layers * kv.B * kv.H_kv;
     size_t R = (size_t)(kv.H_q / kv.H_kv) * w;
-    size_t nch = ((size_t)kv.L_cap + kScoreChunk - 1) / kScoreChunk;
     char *p = (char *)base;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -32,10 +45,9 @@ ScoreWs score_ws_layout(const reco_kv &kv, int w, void *base)
         return r;
     };
     ScoreWs ws;
-    // up to two partials per (unit, chunk, row): the tensor-core pass 1 may split a
-    // chunk's key tiles between two epilogue groups
-    ws.part_m = (float *)take(units * nch * 2 * R * 4);
-    ws.part_z = (float *)take(units * nch * 2 * R * 4);
+    const size_t parts = score_row_parts(kv, w);  // per row
+    ws.part_m = (float *)take(units * parts * R * 4);
+    ws.part_z = (float *)take(units * parts * R * 4);
     ws.rowb = (float *)take(units * R * 4);
     ws.raw = (float *)take(units * (size_t)kv.L_cap * 4);
     ws.ulist = (int32_t *)take(units * 4);
@@ -44,81 +56,138 @@ ScoreWs score_ws_layout(const reco_kv &kv, int w, void *base)
     return ws;
 }
 
-// Pass 1: one thread per window row, its query held in registers; K streamed
-// through shared memory 64 rows at a time.
+// ---------------------------------------------------------------- passes on plain FMAs
+// float32 caches (and bf16 shapes the tensor-core passes do not cover): every product and sum in
+// float32.  Both passes are register-tiled: a CTA holds a tile of 128 keys in shared memory and
+// takes the unit's window rows 64 at a time, each of its 256 threads computing a 4 x 8 block of
+// logits from float4 reads along d (rows ty + 16 i, keys tx + 16 j; the row stride of D + 4 floats
+// keeps the reads of a quarter-warp on different banks).  The CTAs, two per SM so that one loads
+// while the other multiplies, share the call's tiles as the plan deals them.
+//
+// The FMA issue bounds it: a thread's 128 FMAs per four elements of d come with 12 shared-memory
+// reads (43 TFLOP/s; the same with paired FMAs, whose halved instructions bring nothing).  Both
+// passes over 64 units of about 3500 keys, d 128, 192 window rows: 2401 -> 555 us from one key or
+// row per thread, one read per four FMAs and 2048 keys a CTA.
+constexpr int kSimtRows = 64, kSimtThreads = 256;
+
+template <int D> struct SimtSmem {
+    static constexpr int LD = D + 4;  // floats per row
+    static constexpr size_t BYTES = (size_t)(kTile + kSimtRows) * LD * sizeof(float);
+};
+
+// `rows` rows of D elements from src into dst (float32, LD apart), of which `valid` exist; zeros
+// stand for the others.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) score_rowstats_simt(
-    const T *__restrict__ q_win, const T *__restrict__ K, const int32_t *__restrict__ lens, ScoreMask mask,
-    int w, int G, int Hq, int Hkv, int L_cap, int R, int n_chunks, float c2, float *__restrict__ part_m,
+__device__ __forceinline__ void simt_load(float *dst, const T *__restrict__ src, int rows, int valid)
+{
+    constexpr int C = D / 4;  // groups of four elements per row
+#pragma unroll 8
+    for (int e = threadIdx.x; e < rows * C; e += kSimtThreads) {
+        const int r = e / C, c = 4 * (e % C);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < valid) {
+            if constexpr (sizeof(T) == 4) {
+                v = __ldg(reinterpret_cast<const float4 *>(src + (long)r * D + c));
+            } else {
+                const uint2 x = __ldg(reinterpret_cast<const uint2 *>(src + (long)r * D + c));
+                const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.x));
+                const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&x.y));
+                v = make_float4(lo.x, lo.y, hi.x, hi.y);
+            }
+        }
+        *reinterpret_cast<float4 *>(dst + r * SimtSmem<D>::LD + c) = v;
+    }
+}
+
+// s[i][j] = row ty + 16 i of Qs . row tx + 16 j of Ks
+template <int D> __device__ __forceinline__ void simt_logits(const float *Qs, const float *Ks, float (&s)[4][8])
+{
+    constexpr int LD = SimtSmem<D>::LD;
+    const float *q = Qs + (threadIdx.x >> 4) * LD, *k = Ks + (threadIdx.x & 15) * LD;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[i][j] = 0.f;
+#pragma unroll 4
+    for (int c = 0; c < D; c += 4) {
+        float4 a[4], b[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4 *>(q + 16 * i * LD + c);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4 *>(k + 16 * j * LD + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                s[i][j] = fmaf(a[i].x, b[j].x, s[i][j]);
+                s[i][j] = fmaf(a[i].y, b[j].y, s[i][j]);
+                s[i][j] = fmaf(a[i].z, b[j].z, s[i][j]);
+                s[i][j] = fmaf(a[i].w, b[j].w, s[i][j]);
+            }
+    }
+}
+
+// Pass 1: one (max, sum) partial per window row and part_tiles tiles of keys (one CTA's, one after
+// another: the row's thread adds each to the partial).
+template <typename T, int D>
+__global__ void __launch_bounds__(kSimtThreads, 2) score_rowstats_simt(
+    const T *__restrict__ q_win, const T *__restrict__ K, const int32_t *__restrict__ lens, ScoreMask mask, int w, int G,
+    int Hq, int Hkv, int L_cap, int R, int n_parts, int part_tiles, int units, float c2, float *__restrict__ part_m,
     float *__restrict__ part_z, unsigned *err)
 {
-    constexpr int KT = 64;
-    __shared__ __align__(16) float Ks[KT][D];
-    const int chunk = blockIdx.x;
-    const long u = blockIdx.y;
-    const int r = blockIdx.z * blockDim.x + threadIdx.x;
-    const int L = lens[u];
-    if (L < w || L > L_cap) {
-        if (chunk == 0 && blockIdx.z == 0 && threadIdx.x == 0) raise_error(err, ERR_LEN);
-        return;
-    }
-    if (mask.skip(u, L, w, L_cap)) return;
-    const int j0 = chunk * kScoreChunk;
-    const int j1 = min(j0 + kScoreChunk, L);
-    const long lb = u / Hkv;
-    const int h = (int)(u % Hkv);
-    const bool row_ok = r < R;
-    const int g = row_ok ? r / w : 0, t = row_ok ? r % w : 0;
-    const int jmax = L - w + t;
-    float q[D];
-    {
-        const T *qp = q_win + (((lb * Hq) + (long)h * G + g) * w + t) * D;
+    extern __shared__ __align__(16) float smem[];
+    float *Ks = smem, *Qs = smem + kTile * SimtSmem<D>::LD;
+    __shared__ TilePlan plan;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    wait_prior_grid();  // lens, the queries and the cache may come from the previous kernels
+    for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
+        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, false, part_tiles * kTile, skip, nullptr, nullptr, err);
+        for (int e = 0; e < min(kPlanRuns, n_runs - skip); ++e) {
+            const TileRun run = plan.run[e];
+            const T *q = q_win + ((long)(run.u / Hkv) * Hq + (long)(run.u % Hkv) * G) * w * D;
+            for (int t = run.t0; t < run.t0 + run.nt; ++t) {
+                const int j0 = t * kTile;
+                for (int r0 = 0; r0 < R; r0 += kSimtRows) {
+                    __syncthreads();  // the tiles before these have been read
+                    if (r0 == 0) simt_load<T, D>(Ks, K + ((long)run.u * L_cap + j0) * D, kTile, run.L - j0);
+                    simt_load<T, D>(Qs, q + (long)r0 * D, kSimtRows, R - r0);
+                    __syncthreads();
+                    float s[4][8];
+                    simt_logits<D>(Qs, Ks, s);
 #pragma unroll
-        for (int c = 0; c < D; ++c) q[c] = row_ok ? to_float(qp[c]) : 0.f;
-    }
-    float m = -INFINITY, z = 0.f;
-    const T *Kp = K + u * (long)L_cap * D;
-    for (int jt = j0; jt < j1; jt += KT) {
-        const int nk = min(KT, j1 - jt);
-        __syncthreads();
-        for (int e = threadIdx.x; e < KT * D; e += blockDim.x) {
-            int jj = e / D, c = e % D;
-            Ks[jj][c] = jj < nk ? to_float(Kp[(long)(jt + jj) * D + c]) : 0.f;
-        }
-        __syncthreads();
-        if (row_ok) {
-            for (int jj = 0; jj < nk; ++jj) {
-                if (jt + jj > jmax) break;
-                float s = 0.f;
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = r0 + ty + 16 * i;
+                        const int last = min(run.L - 1, run.L - w + r % w);  // the last key this row sees
+                        float m = -INFINITY, z = 0.f;
 #pragma unroll
-                for (int c = 0; c < D; c += 4) {
-                    float4 kv = *reinterpret_cast<const float4 *>(&Ks[jj][c]);
-                    s = fmaf(q[c], kv.x, s);
-                    s = fmaf(q[c + 1], kv.y, s);
-                    s = fmaf(q[c + 2], kv.z, s);
-                    s = fmaf(q[c + 3], kv.w, s);
-                }
-                s *= c2;
-                if (s > m) {
-                    z = z * fast_exp2(m - s) + 1.f;
-                    m = s;
-                } else {
-                    z += fast_exp2(s - m);
+                        for (int j = 0; j < 8; ++j) {
+                            s[i][j] = j0 + tx + 16 * j <= last ? s[i][j] * c2 : -INFINITY;
+                            m = fmaxf(m, s[i][j]);
+                        }
+#pragma unroll
+                        for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                        const float base = m == -INFINITY ? 0.f : m;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) z += fast_exp2(s[i][j] - base);
+#pragma unroll
+                        for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+                        if (tx == 0 && r < R) {
+                            const size_t o = ((size_t)run.u * n_parts + t / part_tiles) * R + r;
+                            if (t % part_tiles) lse_merge(m, z, part_m[o], part_z[o]);
+                            part_m[o] = m;
+                            part_z[o] = z;
+                        }
+                    }
                 }
             }
         }
     }
-    if (row_ok) {
-        size_t o = ((size_t)u * n_chunks + chunk) * R + r;
-        part_m[o] = m;
-        part_z[o] = z;
-    }
 }
 
-// Merge the partials of each row (per_chunk of them for each key chunk, laid out
-// [unit][chunk][per_chunk][R]) into b_r = m_r + log2(Z_r).
+// Merge the partials of each row (`per` of them for each part_keys keys, laid out
+// [unit][n_parts][R]) into b_r = m_r + log2(Z_r).
 __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, int w, int L_cap, int R,
-                              int n_chunks, int per_chunk, const float *__restrict__ part_m,
+                              int n_parts, int part_keys, int per, const float *__restrict__ part_m,
                               const float *__restrict__ part_z, float *__restrict__ rowb, long units)
 {
     wait_prior_grid();  // the partials come from pass 1
@@ -128,9 +197,9 @@ __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, 
     int r = (int)(i % R);
     int L = lens[u];
     if (L < w || L > L_cap || mask.skip(u, L, w, L_cap)) return;
-    int used = ((L + kScoreChunk - 1) / kScoreChunk) * per_chunk;
+    const int used = ((L + part_keys - 1) / part_keys) * per;
     float m = -INFINITY, z = 0.f;
-    const size_t o0 = (size_t)u * n_chunks * per_chunk * R + r;
+    const size_t o0 = (size_t)u * n_parts * R + r;
     constexpr int U = 8;  // partials in flight
     for (int c0 = 0; c0 < used; c0 += U) {
         float pm[U], pz[U];
@@ -239,55 +308,61 @@ __global__ void __launch_bounds__(1024) lse_push_kernel(const float *__restrict_
     if (threadIdx.x == 0) *slot = (s + 1) % slots;
 }
 
-// Pass 2: one thread per candidate key, its key row held in registers; the window
-// queries sit in shared memory and are read by broadcast.
+// Pass 2: every thread's column sums over its rows, added over the row threads at the tile's end.
 template <typename T, int D>
-__global__ void __launch_bounds__(128) score_colsum_simt(
-    const T *__restrict__ q_win, const T *__restrict__ K, const int32_t *__restrict__ lens, ScoreMask mask,
-    int w, int G, int Hq, int Hkv, int L_cap, int R, float c2, const float *__restrict__ rowb,
-    float *__restrict__ raw)
+__global__ void __launch_bounds__(kSimtThreads, 2) score_colsum_simt(
+    const T *__restrict__ q_win, const T *__restrict__ K, const int32_t *__restrict__ lens, ScoreMask mask, int w, int G,
+    int Hq, int Hkv, int L_cap, int R, int units, float c2, const float *__restrict__ rowb, float *__restrict__ raw,
+    int32_t *ulist, int32_t *ucount)
 {
     extern __shared__ __align__(16) float smem[];
-    float *Qs = smem;         // [R][D]
-    float *Bs = smem + R * D; // [R]
-    const int chunk = blockIdx.x;
-    const long u = blockIdx.y;
-    const int L = lens[u];
-    if (L < w || L > L_cap || mask.skip(u, L, w, L_cap)) return;
-    const int nc = L - w;
-    const int j0 = chunk * kScoreChunk;
-    const int j1 = min(j0 + kScoreChunk, nc);
-    if (j0 >= j1) return;
-    const long lb = u / Hkv;
-    const int h = (int)(u % Hkv);
-    for (int e = threadIdx.x; e < R * D; e += blockDim.x) {
-        int rr = e / D, c = e % D;
-        int g = rr / w, t = rr % w;
-        Qs[e] = to_float(q_win[(((lb * Hq) + (long)h * G + g) * w + t) * D + c]);
-    }
-    for (int rr = threadIdx.x; rr < R; rr += blockDim.x) Bs[rr] = rowb[u * R + rr];
-    __syncthreads();
-    const T *Kp = K + u * (long)L_cap * D;
+    float *Ks = smem, *Qs = smem + kTile * SimtSmem<D>::LD;
+    __shared__ TilePlan plan;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const float invG = 1.f / (float)G;
-    for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-        float k[D];
+    wait_prior_grid();  // lens, the normalisers, the queries and the cache may come from the previous kernels
+    for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
+        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, nullptr);
+        for (int e = 0; e < min(kPlanRuns, n_runs - skip); ++e) {
+            const TileRun run = plan.run[e];
+            const int nc = run.L - w;
+            const T *q = q_win + ((long)(run.u / Hkv) * Hq + (long)(run.u % Hkv) * G) * w * D;
+            for (int t = run.t0; t < run.t0 + run.nt; ++t) {
+                const int j0 = t * kTile;
+                float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+                for (int r0 = 0; r0 < R; r0 += kSimtRows) {
+                    float b[4];
 #pragma unroll
-        for (int c = 0; c < D; ++c) k[c] = to_float(Kp[(long)j * D + c]);
-        float acc = 0.f;
-        for (int rr = 0; rr < R; ++rr) {
-            const float *qr = Qs + rr * D;
-            float s = 0.f;
+                    for (int i = 0; i < 4; ++i) {
+                        const int r = r0 + ty + 16 * i;
+                        b[i] = r < R ? rowb[(long)run.u * R + r] : INFINITY;  // a padding row adds 2^-inf = 0
+                    }
+                    __syncthreads();  // the tiles before these have been read
+                    if (r0 == 0) simt_load<T, D>(Ks, K + ((long)run.u * L_cap + j0) * D, kTile, nc - j0);
+                    simt_load<T, D>(Qs, q + (long)r0 * D, kSimtRows, R - r0);
+                    __syncthreads();
+                    float s[4][8];
+                    simt_logits<D>(Qs, Ks, s);
 #pragma unroll
-            for (int c = 0; c < D; c += 4) {
-                float4 qv = *reinterpret_cast<const float4 *>(qr + c);
-                s = fmaf(qv.x, k[c], s);
-                s = fmaf(qv.y, k[c + 1], s);
-                s = fmaf(qv.z, k[c + 2], s);
-                s = fmaf(qv.w, k[c + 3], s);
+                    for (int j = 0; j < 8; ++j)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) sum[j] += fast_exp2(fmaf(s[i][j], c2, -b[i]));
+                }
+                __syncthreads();  // Qs has been read: the warps' sums go there
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    sum[j] += __shfl_xor_sync(0xffffffffu, sum[j], 16);
+                    if (lane < 16) Qs[wid * kTile + tx + 16 * j] = sum[j];
+                }
+                __syncthreads();
+                if (threadIdx.x < kTile && j0 + (int)threadIdx.x < nc) {
+                    float a = 0.f;
+#pragma unroll
+                    for (int k = 0; k < kSimtThreads / 32; ++k) a += Qs[k * kTile + threadIdx.x];
+                    raw[(long)run.u * L_cap + j0 + threadIdx.x] = a * invG;
+                }
             }
-            acc += fast_exp2(fmaf(s, c2, -Bs[rr]));
         }
-        raw[u * L_cap + j] = acc * invG;
     }
 }
 
@@ -432,40 +507,42 @@ cudaError_t launch_score_tc_pass1(const reco_kv &kv, const void *q_win, const in
 cudaError_t launch_score_tc_pass2(const reco_kv &kv, const void *q_win, const int32_t *lens, const ScoreMask &mask,
                                   int w, float c2, const ScoreWs &ws, const float *row_lse, unsigned *err,
                                   cudaStream_t s, bool *used);
-bool score_tc_supported(const reco_kv &kv, int w);
 int score_tc_pass1_groups(int R);
 
-// SIMT passes; with pass1 false the row normalisers are already in ws.rowb.
+// Passes on plain FMAs; with pass1 false the row normalisers are already in ws.rowb.  A masked
+// call's pass 2 also lists the units it scored in ws.ulist / ws.ucount.
 template <typename T, int D>
 static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *lens, ScoreMask mask, int w,
                               float c2, const ScoreWs &ws, unsigned *err, cudaStream_t s, bool pass1 = true)
 {
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
     const int G = kv.H_q / kv.H_kv, R = G * w;
-    const int nch = (kv.L_cap + kScoreChunk - 1) / kScoreChunk;
+    const long tiles = units * ((kv.L_cap + kTile - 1) / kTile);
+    const dim3 grid((unsigned)std::min(tiles, 2L * device_sm_count())), block(kSimtThreads);
+    constexpr size_t smem = SimtSmem<D>::BYTES;
     const T *K = (const T *)kv.k;
     cudaError_t e = cudaSuccess;
     if (pass1) {
-        int bx = R < 256 ? ((R + 31) / 32) * 32 : 256;
-        dim3 g1(nch, (unsigned)units, (R + bx - 1) / bx);
-        score_rowstats_simt<T, D><<<g1, bx, 0, s>>>(q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap, R,
-                                                    nch, c2, ws.part_m, ws.part_z, err);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        long n = units * R;
-        score_combine<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(lens, mask, w, kv.L_cap, R, nch, 1, ws.part_m,
-                                                                  ws.part_z, ws.rowb, units);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const int n_parts = score_row_parts(kv, w), part_tiles = simt_part_tiles(kv, w);
+        e = cudaFuncSetAttribute(score_rowstats_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        e = launch_pdl(score_rowstats_simt<T, D>, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv,
+                       kv.L_cap, R, n_parts, part_tiles, (int)units, c2, ws.part_m, ws.part_z, err);
+        if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_pdl(score_combine, dim3((unsigned)((units * R + 255) / 256)), dim3(256), 0, s, lens, mask, w,
+                       kv.L_cap, R, n_parts, part_tiles * kTile, 1, (const float *)ws.part_m, (const float *)ws.part_z, ws.rowb,
+                       units);
+        if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    size_t smem = ((size_t)R * D + R) * sizeof(float);
-    e = cudaFuncSetAttribute(score_colsum_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+    e = cudaFuncSetAttribute(score_colsum_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    score_colsum_simt<T, D><<<dim3(nch, (unsigned)units), 128, smem, s>>>(
-        q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap, R, c2, ws.rowb, ws.raw);
-    return cudaGetLastError();
+    e = launch_pdl(score_colsum_simt<T, D>, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap,
+                   R, (int)units, c2, (const float *)ws.rowb, ws.raw, mask.keep ? ws.ulist : nullptr,
+                   mask.keep ? ws.ucount : nullptr);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Largest R*D the SIMT pass 2 keeps in shared memory.
+// Largest R*D (and R more) the calls outside the tensor-core passes accept.
 constexpr size_t kSimtMaxQ = 200 * 1024 / 4;
 
 bool score_shape_supported(const reco_kv &kv, int w)
@@ -525,8 +602,8 @@ cudaError_t launch_score(const reco_kv &kv, const void *q_win, const int32_t *le
             const int R = (kv.H_q / kv.H_kv) * w;
             const int nch = (kv.L_cap + kScoreChunk - 1) / kScoreChunk;
             e = launch_pdl(score_combine, dim3((unsigned)((units * R + 255) / 256)), dim3(256), 0, s, lens, mask, w,
-                           kv.L_cap, R, nch, score_tc_pass1_groups(R), (const float *)ws.part_m,
-                           (const float *)ws.part_z, ws.rowb, units);
+                           kv.L_cap, R, nch * score_tc_pass1_groups(R), kScoreChunk, score_tc_pass1_groups(R),
+                           (const float *)ws.part_m, (const float *)ws.part_z, ws.rowb, units);
             if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
             bool used2 = false;
             e = launch_score_tc_pass2(kv, q_win, lens, mask, w, c2, ws, nullptr, err, s, &used2);

@@ -59,3 +59,19 @@ def test_more_units_than_one_plan_round():
 def test_pool_tiles(dtype, L, pool):
     wl = W.WORKLOADS["7b"].reduced(layers=1, batch=1, h_q=4, h_kv=2, d=64, L=L, decode_steps=0, w=16, dtype=dtype)
     _check(wl, np.array([[[L, 4096 + 17 if L < 8000 else 4111]]], np.int32), pool, [(0, 0, 0), (0, 0, 1)])
+
+
+# plain-FMA passes: rows below, at and past a 64-row tile, units shorter than one key tile, ragged
+@pytest.mark.parametrize("G,w,d", [(1, 5, 64), (4, 16, 128), (13, 5, 128), (6, 32, 128), (10, 39, 128), (12, 64, 64)])
+def test_f32_row_counts(G, w, d):
+    wl = W.WORKLOADS["7b"].reduced(layers=2, batch=2, h_q=2 * G, h_kv=2, d=d, L=1500, decode_steps=5, w=w, dtype="f32")
+    rng = np.random.default_rng(G * 100 + w)
+    lens = rng.integers(w, 1506, (2, 2, 2)).astype(np.int32)
+    lens[0, 0, 0], lens[0, 1, 1], lens[1, 1, 1] = 1505, 128 + w, w + 1
+    _check(wl, lens, 7, [(0, 0, 0), (0, 1, 1), (1, 0, 0), (1, 1, 1)])
+
+
+def test_bf16_rows_beyond_the_tensor_cores():
+    """R = 760 window rows at d = 64: the plain-FMA passes read bf16 rows."""
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=2, h_q=38, h_kv=2, d=64, L=700, decode_steps=0, w=40)
+    _check(wl, np.array([[[700, 333], [40, 168]]], np.int32), 7, [(0, 0, 0), (0, 0, 1), (0, 1, 1)])
