@@ -1,29 +1,34 @@
 // decode.cu -- decode attention over the ragged compacted cache, the per-token
 // attention whose cost the compression lowers (Sec. 1; Sec. 2.2; Sec. 4.2).
 //
-// bf16 path (decode_tma): a persistent split-K flash-decode, one CTA of 8 warps per
-// SM (for long work 4 of them, each with a ring twice as deep).  Every CTA first
-// builds the same work plan from lens: the prefix sum of 16-key blocks per unit, with
-// the blocks of all units laid end to end and cut into one equal contiguous range per
-// warp (a stream-K split: balanced to one block, no work queue).  A call with more units
-// than one plan holds runs as consecutive launches over contiguous unit ranges.
-// When no unit is long enough to be cut, the units are instead sorted by length and
-// dealt whole to the warps in snake order (longest first).
-// An item's keys stream from HBM in 16-key blocks: one lane issues TMA tensor copies
-// (128-byte swizzled 16 x 64 tiles of K and V) into the warp's 3-stage ring and the
-// warp waits on the stage's mbarrier (bounded).  QK^T and PV run on mma.sync
-// m16n8k16 (bf16 in, fp32 accumulate) with the G <= 8 query heads of the KV head
-// packed into one MMA tile.  The head dimension is permuted consistently on the Q
-// and K sides (and on the V and output sides) so that each thread's fragments are
-// whole 16-byte chunks, and the swizzle makes every fragment read conflict-free.  A
-// unit split over several items writes partial (max, sum, output) triples; the last
+// decode_stream: a persistent split-K flash-decode, one CTA of 8 warps per SM (for long
+// bf16 work 4 of them, each with a ring twice as deep).  Every CTA first builds the same
+// work plan from lens: the prefix sum of blocks of keys per unit, with the blocks of all
+// units laid end to end and cut into one equal contiguous range per warp (a stream-K
+// split: balanced to one block, no work queue).  A call with more units than one plan
+// holds runs as consecutive launches over contiguous unit ranges.  When no unit is long
+// enough to be cut, the units are instead sorted by length and dealt whole to the warps in
+// snake order (longest first).  An item's keys stream from HBM in blocks of 8 KB (at d =
+// 128): one lane issues bulk copies of K and V into the warp's 3-stage ring and the warp
+// waits on the stage's mbarrier (bounded).  What a warp does with a block is a template
+// parameter, a block consumer.
+//   bf16: blocks of 16 keys by TMA tensor copies (128-byte swizzled 16 x 64 tiles); QK^T
+//   and PV on mma.sync m16n8k16 (fp32 accumulate), up to 16 query heads.  The head
+//   dimension is permuted consistently on the Q and K sides (and on the V and output
+//   sides) so that each thread's fragments are whole 16-byte chunks, and the swizzle makes
+//   every fragment read conflict-free.  Heads 9 to 16 of a unit fill the QK tile's other
+//   eight rows: one pass over the block instead of two units of half the heads (28 x 4 x 4
+//   units of 2000 to 4100 rows, 16 heads: 226 -> 157 us).
+//   float32: blocks of 8 keys, plain FMAs (28 x 4 x 2 units of 800 to 1500 rows, 6 heads,
+//   from one CTA per unit that took its keys one by one: 516 -> 67 us).
+// A unit split over several items writes partial (max, sum, output) triples; the last
 // item to finish (atomic ticket, no waiting) merges them.  The counters live in the
 // caller's workspace, zero-filled before its first use; each launch clears what it
 // counted, so no reset runs between launches.  The appended token (k_new, v_new) is
 // read from the inputs and written into the cache by the warp that covers its index;
 // the last warp of the grid to finish advances lens.
 //
-// float32 path (decode_simt): one CTA per unit, four warps over the keys, G <= 16.
+// decode_simt serves bf16 calls for which no tensor map can be made.
 #include <cuda.h>
 
 #include <algorithm>
@@ -70,13 +75,12 @@ struct DecodeArgs {
     int units, Hq, Hkv, G, L_cap, append, out_bf16;
     float c2;  // scale * log2(e)
     unsigned *err;
-    int hs, gv;       // TMA path: hs virtual units of gv (<= 8) query heads per unit (G > 8: hs = 2)
+    int gv;           // query heads per virtual unit (half of G where a unit runs as two)
     float *ring;      // or nullptr: lse rows ring[*slot] and ring[*slot + slots], each [nq]
     long long *slot;  // device ring row, advanced by one (mod slots) per launch
     int slots;
     long long nq;     // query heads of the launch (layers * B * H_q)
     void *qring;      // or nullptr: [nq][slots][D] of q's dtype, row *slot of every head gets its query
-    int q_bytes;      // bytes per element of q
     long long nq_rows;  // query heads of this launch (nq, or a part of it when the units are split)
     int advance;        // this launch advances *slot (the last of a split launch's parts)
 };
@@ -124,7 +128,7 @@ __device__ __forceinline__ bool unit_ok(int L, int L_cap, int append)
     return L >= 0 && L <= L_cap && (!append || L < L_cap);
 }
 
-template <typename T> __device__ __forceinline__ void store_out(void *out, bool bf16, size_t i, float v)
+__device__ __forceinline__ void store_out(void *out, bool bf16, size_t i, float v)
 {
     if (bf16)
         reinterpret_cast<__nv_bfloat16 *>(out)[i] = __float2bfloat16_rn(v);
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(128) decode_simt(DecodeArgs a)
             }
         }
         const size_t row = (size_t)(lb * a.Hq + (long)h * G + g);
-        store_out<T>(a.out, a.out_bf16, row * D + dd, Ls > 0.f ? O / Ls : 0.f);
+        store_out(a.out, a.out_bf16, row * D + dd, Ls > 0.f ? O / Ls : 0.f);
         if (dd == 0) put_lse(a, rs, row, Ls > 0.f ? (M + log2f(Ls)) * kLn2 : -INFINITY);
     }
     if (ok && a.append) {
@@ -228,7 +232,7 @@ __global__ void __launch_bounds__(128) decode_simt(DecodeArgs a)
     }
 }
 
-// ---------------------------------------------------------------- tensor-core path
+// ---------------------------------------------------------------- streamed path
 __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1)
 {
@@ -268,45 +272,517 @@ constexpr int kMinBlocksPerWarp = 4;         // fewer working warps rather than 
 constexpr int kMaxWholeBlocks = 16;          // units of at most this many blocks are never cut
 constexpr int kDeepBlocksPerWarp = 64;       // from this many blocks per warp, half the warps with deep rings
 
-template <int D> struct TmaLayout {
-    static constexpr int HALVES = D / 64;             // 128-byte boxes per row
-    static constexpr int TILE = 16 * 128;             // one 16-row box
-    static constexpr int STAGE = 4 * HALVES * 16 * 64; // K boxes then V boxes (bytes)
+constexpr int kStageBytes128 = 8192;         // a block of K and V rows at d = 128 (half of it at d = 64)
+
+template <int D> struct RingLayout {
+    static constexpr int STAGE = kStageBytes128 * D / 128;
     static constexpr int RING = kDecodeWarps * kDecodeStages * STAGE;
 };
 
-// the largest plan fits beside the d = 128 ring (227 KB per CTA, about 1 KB of it static)
-static_assert(1024 + TmaLayout<128>::RING + (kMaxTmaUnits + 1) * 4 + 1024 <= 227 * 1024, "decode smem budget");
-static_assert((kMaxTmaUnits + 32 + (kMaxWholeBlocks + 1) * kDecodeWarps * 32) * 4 <= TmaLayout<64>::RING,
+// the largest plan fits beside the d = 128 ring (227 KB per CTA, about 1 KB of it static, for
+// float32 about 3 KB)
+constexpr int kMaxF32Units = kMaxTmaUnits - 1024;
+static_assert(1024 + RingLayout<128>::RING + (kMaxTmaUnits + 1) * 4 + 1024 <= 227 * 1024, "decode smem budget");
+static_assert(1024 + RingLayout<128>::RING + (kMaxF32Units + 1) * 4 + 4 * 1024 <= 227 * 1024, "decode smem budget");
+static_assert((kMaxTmaUnits + 32 + (kMaxWholeBlocks + 1) * kDecodeWarps * 32) * 4 <= RingLayout<64>::RING,
               "lengths and the sort counters are staged in the ring");
 
 template <int D>
-size_t tma_smem_bytes(int units)
+size_t ring_smem_bytes(int units)
 {
-    return 1024 + (size_t)TmaLayout<D>::RING + (size_t)(units + 1) * sizeof(int);
+    return 1024 + (size_t)RingLayout<D>::RING + (size_t)(units + 1) * sizeof(int);
 }
 
 // Byte offset of 16-byte chunk ch (0..7) of row rr inside a 128B-swizzled 16-row box.
 __device__ __forceinline__ uint32_t swz(int rr, int ch) { return rr * 128 + ((ch ^ (rr & 7)) << 4); }
 
-template <int D, int HS>
+// A block consumer holds one item's queries, running (max, sum) and output in a warp's registers
+// and takes the item's keys in blocks of KB rows from the warp's ring.  It says how a block is
+// copied (load), where a 16-byte chunk of a row lies in a stage (chunk), and how results leave.
+
+// bf16: QK^T and PV run on mma.sync m16n8k16 with NT * 8 query heads per unit.  The QK tile has
+// 16 query rows: heads 0-7 fill its first eight, heads 8-15 (NT = 2) the others, which cost the
+// product nothing more; PV takes one 8-head column tile per NT.
+template <int D_, int NT_> struct Bf16Block {
+    static constexpr int D = D_, HS = 1, NT = NT_, KB = 16, GM = 8 * NT;
+    static constexpr int ROW = 2 * D, HALVES = D / 64, TILE = 16 * 128, MT = D / 16;
+    static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = 0;
+    static constexpr bool TENSOR_MAPS = true, PREFETCH_Q = NT == 1;
+    // half the warps with deeper rings for long work: up to eight heads a block leaves a warp
+    // waiting for data; with sixteen its arithmetic wants all the warps (160 against 155 us)
+    static constexpr bool DEEP = NT == 1;
+
+    uint32_t qa[D / 16][2 * NT], qn[PREFETCH_Q ? D / 16 : 1][2 * NT];
+    float o[NT][MT][4], m[NT], l[NT];
+    const __nv_bfloat16 *q_src = nullptr;
+    int nh_src = 0;
+    const int g, c;
+
+    __device__ __forceinline__ Bf16Block(int lane, float *) : g(lane >> 2), c(lane & 3) {}
+
+    __device__ static __forceinline__ uint32_t chunk(int row, int ch) { return (ch >> 3) * TILE + swz(row, ch & 7); }
+
+    // 128-byte swizzled 16 x 64 boxes of K, then of V (whole boxes: rows past the item are masked)
+    __device__ static __forceinline__ void load(uint32_t dst, uint32_t bar, const CUtensorMap *tmK,
+                                                const CUtensorMap *tmV, const DecodeArgs &a, int pu, int k, int,
+                                                uint64_t policy)
+    {
+        const int y = pu * a.L_cap + k;
+        mbar_expect_tx(bar, 2 * HALVES * TILE);
+#pragma unroll
+        for (int hh = 0; hh < HALVES; ++hh) {
+            tma_load_2d_hint(dst + hh * TILE, tmK, 64 * hh, y, bar, policy);
+            tma_load_2d_hint(dst + (HALVES + hh) * TILE, tmV, 64 * hh, y, bar, policy);
+        }
+    }
+
+    // Q fragments, the head dim permuted to match the K chunks: k-step j = 4*hh + 2*e + half takes
+    // elements 64*hh + 16c + 8e + 4*half + {0,1} and + {2,3} (of rows g, then g + 8)
+    __device__ __forceinline__ void fragments(const __nv_bfloat16 *q, int nh, uint32_t (&f)[D / 16][2 * NT]) const
+    {
+#pragma unroll
+        for (int hh = 0; hh < HALVES; ++hh)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    uint4 wv = make_uint4(0, 0, 0, 0);
+                    if (g + 8 * n < nh) wv = *reinterpret_cast<const uint4 *>(q + (g + 8 * n) * D + 64 * hh + 16 * c + 8 * e);
+                    const int j = 4 * hh + 2 * e;
+                    f[j][n] = wv.x;
+                    f[j][NT + n] = wv.y;
+                    f[j + 1][n] = wv.z;
+                    f[j + 1][NT + n] = wv.w;
+                }
+    }
+
+    // the queries of the item that start() will begin
+    __device__ __forceinline__ void load_q(const void *q, long qrow, int nh)
+    {
+        q_src = reinterpret_cast<const __nv_bfloat16 *>(q) + qrow * D;
+        nh_src = nh;
+        if constexpr (PREFETCH_Q) fragments(q_src, nh, qn);
+    }
+
+    __device__ __forceinline__ void start()
+    {
+        if constexpr (PREFETCH_Q) {
+#pragma unroll
+            for (int j = 0; j < D / 16; ++j)
+#pragma unroll
+                for (int n = 0; n < 2 * NT; ++n) qa[j][n] = qn[j][n];
+        } else {
+            fragments(q_src, nh_src, qa);
+        }
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            m[n] = -INFINITY;
+            l[n] = 0.f;
+#pragma unroll
+            for (int t = 0; t < MT; ++t) o[n][t][0] = o[n][t][1] = o[n][t][2] = o[n][t][3] = 0.f;
+        }
+    }
+
+    __device__ __forceinline__ void consume(uint32_t Ks, uint32_t Vs, int kb, int k1, float c2)
+    {
+        // four accumulators (keys 0-7 / 8-15, even / odd k-steps): dependent MMA chains
+        // of D/32 instead of D/16
+        float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
+        float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int hh = 0; hh < HALVES; ++hh)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint4 ka = lds_u4(Ks + hh * TILE + swz(g, 2 * c + e));
+                const uint4 kc = lds_u4(Ks + hh * TILE + swz(8 + g, 2 * c + e));
+                const int j = 4 * hh + 2 * e;
+                const uint32_t a1 = NT == 2 ? qa[j][1 % (2 * NT)] : 0u, a3 = NT == 2 ? qa[j][3 % (2 * NT)] : 0u;
+                const uint32_t b1 = NT == 2 ? qa[j + 1][1 % (2 * NT)] : 0u, b3 = NT == 2 ? qa[j + 1][3 % (2 * NT)] : 0u;
+                mma_bf16(s0, qa[j][0], a1, qa[j][NT], a3, ka.x, ka.y);
+                mma_bf16(s1, qa[j][0], a1, qa[j][NT], a3, kc.x, kc.y);
+                mma_bf16(t0, qa[j + 1][0], b1, qa[j + 1][NT], b3, ka.z, ka.w);
+                mma_bf16(t1, qa[j + 1][0], b1, qa[j + 1][NT], b3, kc.z, kc.w);
+            }
+        uint32_t ph[NT][2], pl[NT][2];
+        const int kA = kb + 2 * c, kB = kb + 8 + 2 * c;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            // scores of query g + 8n for keys kb+2c, kb+2c+1, kb+8+2c, kb+9+2c
+            const float x0 = (kA < k1) ? (s0[2 * n] + t0[2 * n]) * c2 : -INFINITY;
+            const float x1 = (kA + 1 < k1) ? (s0[2 * n + 1] + t0[2 * n + 1]) * c2 : -INFINITY;
+            const float x2 = (kB < k1) ? (s1[2 * n] + t1[2 * n]) * c2 : -INFINITY;
+            const float x3 = (kB + 1 < k1) ? (s1[2 * n + 1] + t1[2 * n + 1]) * c2 : -INFINITY;
+            float mb = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3));
+            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
+            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
+            // Lazy rescale: a row's reference max m moves only when a block max exceeds it
+            // by more than 2^kLazyLog2, so probabilities against a stale m stay <= 2^8
+            // (exact in fp32, and the bf16 hi + lo split keeps 16 bits of them); the
+            // output rescale below then runs on few blocks.  m, l and o stay consistent, so
+            // o / l and lse = m + log2 l are the same quantities as with an exact max.
+            const bool grow = mb > m[n] + kLazyLog2;
+            if (__any_sync(0xffffffffu, grow)) {
+                const float mn = grow ? mb : m[n];
+                const float alpha = grow ? fast_exp2(m[n] - mn) : 1.f;  // m = -inf gives 0
+                l[n] *= alpha;
+                m[n] = mn;
+                const float al0 = __shfl_sync(0xffffffffu, alpha, (2 * c) * 4);
+                const float al1 = __shfl_sync(0xffffffffu, alpha, (2 * c + 1) * 4);
+#pragma unroll
+                for (int t = 0; t < MT; ++t) {
+                    o[n][t][0] *= al0;
+                    o[n][t][1] *= al1;
+                    o[n][t][2] *= al0;
+                    o[n][t][3] *= al1;
+                }
+            }
+            const float base = (m[n] == -INFINITY) ? 0.f : m[n];
+            const float p0 = fast_exp2(x0 - base), p1 = fast_exp2(x1 - base);
+            const float p2 = fast_exp2(x2 - base), p3 = fast_exp2(x3 - base);
+            l[n] += (p0 + p1) + (p2 + p3);
+            // P enters the PV product as bf16 hi + lo parts (two MMAs), which keeps about
+            // 16 significant bits of each probability instead of 8.
+            split_bf16(p0, p1, ph[n][0], pl[n][0]);
+            split_bf16(p2, p3, ph[n][1], pl[n][1]);
+        }
+#pragma unroll
+        for (int hh = 0; hh < HALVES; ++hh) {
+            const uint4 v0 = lds_u4(Vs + hh * TILE + swz(2 * c, g));
+            const uint4 v1 = lds_u4(Vs + hh * TILE + swz(2 * c + 1, g));
+            const uint4 v2 = lds_u4(Vs + hh * TILE + swz(2 * c + 8, g));
+            const uint4 v3 = lds_u4(Vs + hh * TILE + swz(2 * c + 9, g));
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const uint32_t W0 = word(v0, x), W1 = word(v1, x), W2 = word(v2, x), W3 = word(v3, x);
+                const uint32_t A0 = __byte_perm(W0, W1, 0x5410), A1 = __byte_perm(W0, W1, 0x7632);
+                const uint32_t A2 = __byte_perm(W2, W3, 0x5410), A3 = __byte_perm(W2, W3, 0x7632);
+#pragma unroll
+                for (int n = 0; n < NT; ++n) {
+                    mma_bf16(o[n][4 * hh + x], A0, A1, A2, A3, ph[n][0], ph[n][1]);
+                    mma_bf16(o[n][4 * hh + x], A0, A1, A2, A3, pl[n][0], pl[n][1]);
+                }
+            }
+        }
+    }
+
+    __device__ __forceinline__ void finish()
+    {
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            l[n] += __shfl_xor_sync(0xffffffffu, l[n], 1);
+            l[n] += __shfl_xor_sync(0xffffffffu, l[n], 2);
+        }
+    }
+
+    template <typename F> __device__ __forceinline__ void each_lse(int G, F f) const
+    {
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
+            if (c == 0 && g + 8 * n < G) f(g + 8 * n, m[n], l[n]);
+    }
+
+    __device__ __forceinline__ void store(void *out, bool bf16, long qrow0, int G) const
+    {
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const int q0 = 8 * n + 2 * c, q1 = q0 + 1;
+            const float l0 = __shfl_sync(0xffffffffu, l[n], 8 * c), l1 = __shfl_sync(0xffffffffu, l[n], 8 * c + 4);
+            const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
+#pragma unroll
+            for (int hh = 0; hh < HALVES; ++hh) {
+                const long d0 = 64 * hh + 8 * g;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const float *v = o[n][4 * hh + x];
+                    if (q0 < G) {
+                        store_out(out, bf16, (qrow0 + q0) * D + d0 + 2 * x, v[0] * inv0);
+                        store_out(out, bf16, (qrow0 + q0) * D + d0 + 2 * x + 1, v[2] * inv0);
+                    }
+                    if (q1 < G) {
+                        store_out(out, bf16, (qrow0 + q1) * D + d0 + 2 * x, v[1] * inv1);
+                        store_out(out, bf16, (qrow0 + q1) * D + d0 + 2 * x + 1, v[3] * inv1);
+                    }
+                }
+            }
+        }
+    }
+
+    __device__ __forceinline__ void store_partial(float *po, int G) const
+    {
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+            const int q0 = 8 * n + 2 * c, q1 = q0 + 1;
+#pragma unroll
+            for (int hh = 0; hh < HALVES; ++hh) {
+                const int d0 = 64 * hh + 8 * g;
+                const float(*v)[4] = &o[n][4 * hh];
+                if (q0 < G) {
+                    float4 *dst = reinterpret_cast<float4 *>(po + (size_t)q0 * D + d0);
+                    dst[0] = make_float4(v[0][0], v[0][2], v[1][0], v[1][2]);
+                    dst[1] = make_float4(v[2][0], v[2][2], v[3][0], v[3][2]);
+                }
+                if (q1 < G) {
+                    float4 *dst = reinterpret_cast<float4 *>(po + (size_t)q1 * D + d0);
+                    dst[0] = make_float4(v[0][1], v[0][3], v[1][1], v[1][3]);
+                    dst[1] = make_float4(v[2][1], v[2][3], v[3][1], v[3][3]);
+                }
+            }
+        }
+    }
+};
+
+// float32: plain FMAs in float32 throughout, GT >= G (or half of G, HS = 2) query heads.  In QK^T
+// lane (kq = lane / 8, part = lane % 8) holds D / 8 elements of every head's query (32-element
+// groups, four at part * 4) and multiplies them with keys kq and kq + 4 of the block; the eight
+// parts are then added by halving exchanges that leave each (key, head) sum in one lane.  In PV a
+// lane owns D / 32 columns of every head's output and takes the probabilities from shared memory.
+template <int D_, int GT_, int HS_> struct F32Block {
+    static constexpr int D = D_, HS = HS_, KB = 8, GM = GT_, GT = GT_, E = D / 32, QE = D / 8;
+    static constexpr int ROW = 4 * D;
+    static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = KB * GT;
+    static constexpr bool TENSOR_MAPS = false;
+    static constexpr bool DEEP = false;  // bound by its arithmetic: all the warps (93 against 70 us)
+    static constexpr int VPL = GT == 8 ? 2 : (GT == 6 ? 3 : 1);  // (key, head) sums per lane
+
+    float q[GT][QE], o[GT][E], m[VPL], l[VPL];
+    const float *q_src = nullptr;
+    int nh_src = 0;
+    float *const p_sm;  // [KB][GT] probabilities of the block
+    const int lane;
+
+    __device__ __forceinline__ F32Block(int lane_, float *scratch) : p_sm(scratch), lane(lane_) {}
+
+    __device__ static __forceinline__ uint32_t chunk(int row, int ch) { return row * ROW + ch * 16; }
+
+    // `rows` rows of K, then of V, each one contiguous copy (none when only the appended row is left)
+    __device__ static __forceinline__ void load(uint32_t dst, uint32_t bar, const CUtensorMap *, const CUtensorMap *,
+                                                const DecodeArgs &a, int pu, int k, int rows, uint64_t policy)
+    {
+        const uint32_t bytes = (uint32_t)max(rows, 0) * ROW;
+        mbar_expect_tx(bar, 2 * bytes);
+        if (bytes == 0) return;
+        const size_t off = ((size_t)pu * a.L_cap + k) * ROW;
+        bulk_load_hint(dst, static_cast<const char *>(a.K) + off, bytes, bar, policy);
+        bulk_load_hint(dst + KB * ROW, static_cast<const char *>(a.V) + off, bytes, bar, policy);
+    }
+
+    __device__ __forceinline__ void load_q(const void *qp, long qrow, int nh)
+    {
+        q_src = reinterpret_cast<const float *>(qp) + qrow * D;
+        nh_src = nh;
+    }
+
+    __device__ __forceinline__ void start()
+    {
+#pragma unroll
+        for (int g = 0; g < GT; ++g) {
+#pragma unroll
+            for (int i = 0; i < QE / 4; ++i) {
+                float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (g < nh_src) x = *reinterpret_cast<const float4 *>(q_src + (long)g * D + 32 * i + 4 * (lane & 7));
+                q[g][4 * i] = x.x;
+                q[g][4 * i + 1] = x.y;
+                q[g][4 * i + 2] = x.z;
+                q[g][4 * i + 3] = x.w;
+            }
+#pragma unroll
+            for (int e = 0; e < E; ++e) o[g][e] = 0.f;
+        }
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            m[v] = -INFINITY;
+            l[v] = 0.f;
+        }
+    }
+
+    // the lane (of kq = 0, first key) and its value that hold head g after the exchanges
+    __device__ static __forceinline__ constexpr int lane_of(int g)
+    {
+        return GT == 8 ? g >> 1 : (GT == 6 ? 2 * (g / 3) : (GT == 4 ? g : 2 * g));
+    }
+    __device__ static __forceinline__ constexpr int value_of(int g) { return GT == 8 ? g & 1 : (GT == 6 ? g % 3 : 0); }
+    __device__ __forceinline__ int head_of(int v) const
+    {
+        return GT == 8 ? 2 * (lane & 3) + v : (GT == 4 ? lane & 3 : ((lane >> 1) & 1) * VPL + v);
+    }
+
+    // Halving exchange over lane bit `bit`: of 2N partial sums this lane keeps the lower N (bit
+    // clear) or the upper N, each with its partner's added.
+    template <int N> __device__ __forceinline__ void halve(float *s, int bit) const
+    {
+        const bool up = lane & bit;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const float send = up ? s[i] : s[i + N];
+            const float keep = up ? s[i + N] : s[i];
+            s[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+        }
+    }
+
+    __device__ __forceinline__ void consume(uint32_t Ks, uint32_t Vs, int kb, int k1, float c2)
+    {
+        float s[2 * GT];  // keys kq, then kq + 4
+#pragma unroll
+        for (int i = 0; i < 2 * GT; ++i) s[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const uint32_t row = Ks + ((lane >> 3) + 4 * k) * ROW + (lane & 7) * 16;
+#pragma unroll
+            for (int i = 0; i < QE / 4; ++i) {
+                const float4 x = lds_f4(row + 128 * i);
+#pragma unroll
+                for (int g = 0; g < GT; ++g) {
+                    float t = s[k * GT + g];
+                    t = fmaf(q[g][4 * i], x.x, t);
+                    t = fmaf(q[g][4 * i + 1], x.y, t);
+                    t = fmaf(q[g][4 * i + 2], x.z, t);
+                    s[k * GT + g] = fmaf(q[g][4 * i + 3], x.w, t);
+                }
+            }
+        }
+        halve<GT>(s, 4);      // lane bit 2: the key
+        halve<GT / 2>(s, 2);  // bit 1: the head's high bit
+        if constexpr (GT % 4 == 0) {
+            halve<GT / 4>(s, 1);
+        } else {  // both lanes keep the sums
+#pragma unroll
+            for (int v = 0; v < VPL; ++v) s[v] += __shfl_xor_sync(0xffffffffu, s[v], 1);
+        }
+        const int kk = (lane >> 3) + (lane & 4);  // this lane's key of the block
+        float x[VPL], mb[VPL];
+        bool any = false;
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            x[v] = kb + kk < k1 ? s[v] * c2 : -INFINITY;
+            mb[v] = x[v];
+#pragma unroll
+            for (int o2 = 4; o2 <= 16; o2 <<= 1) mb[v] = fmaxf(mb[v], __shfl_xor_sync(0xffffffffu, mb[v], o2));
+            any |= mb[v] > m[v] + kLazyLog2;
+        }
+        if (__any_sync(0xffffffffu, any)) {  // lazy rescale, as in the bf16 consumer
+            float al[VPL];
+#pragma unroll
+            for (int v = 0; v < VPL; ++v) {
+                const float mn = mb[v] > m[v] + kLazyLog2 ? mb[v] : m[v];
+                al[v] = mn == m[v] ? 1.f : fast_exp2(m[v] - mn);  // m = -inf gives 0
+                l[v] *= al[v];
+                m[v] = mn;
+            }
+#pragma unroll
+            for (int g = 0; g < GT; ++g) {
+                const float f = __shfl_sync(0xffffffffu, al[value_of(g)], lane_of(g));
+#pragma unroll
+                for (int e = 0; e < E; ++e) o[g][e] *= f;
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            const float p = fast_exp2(x[v] - (m[v] == -INFINITY ? 0.f : m[v]));
+            l[v] += p;
+            p_sm[kk * GT + head_of(v)] = p;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+            float p[GT], x[E];
+            if constexpr (GT % 4 == 0) {
+#pragma unroll
+                for (int g = 0; g < GT; g += 4) {
+                    const float4 f = *reinterpret_cast<const float4 *>(p_sm + k * GT + g);
+                    p[g] = f.x;
+                    p[g + 1] = f.y;
+                    p[g + 2] = f.z;
+                    p[g + 3] = f.w;
+                }
+            } else {
+#pragma unroll
+                for (int g = 0; g < GT; g += 2) {
+                    const float2 f = *reinterpret_cast<const float2 *>(p_sm + k * GT + g);
+                    p[g] = f.x;
+                    p[g + 1] = f.y;
+                }
+            }
+            if constexpr (E == 4) {
+                const float4 f = lds_f4(Vs + k * ROW + lane * 16);
+                x[0] = f.x;
+                x[1] = f.y;
+                x[2] = f.z;
+                x[3] = f.w;
+            } else {
+                const float2 f = lds_f2(Vs + k * ROW + lane * 8);
+                x[0] = f.x;
+                x[1] = f.y;
+            }
+#pragma unroll
+            for (int g = 0; g < GT; ++g)
+#pragma unroll
+                for (int e = 0; e < E; ++e) o[g][e] = fmaf(p[g], x[e], o[g][e]);
+        }
+    }
+
+    __device__ __forceinline__ void finish()
+    {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v)
+#pragma unroll
+            for (int o2 = 4; o2 <= 16; o2 <<= 1) l[v] += __shfl_xor_sync(0xffffffffu, l[v], o2);
+        __syncwarp();  // the probabilities have been read
+    }
+
+    template <typename F> __device__ __forceinline__ void each_lse(int G, F f) const
+    {
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            const int g = head_of(v);
+            if (lane == lane_of(g) && g < G) f(g, m[v], l[v]);
+        }
+    }
+
+    __device__ __forceinline__ void store(void *out, bool bf16, long qrow0, int G) const
+    {
+#pragma unroll
+        for (int g = 0; g < GT; ++g) {
+            const float lg = __shfl_sync(0xffffffffu, l[value_of(g)], lane_of(g));
+            if (g < G) {
+                const float inv = lg > 0.f ? 1.f / lg : 0.f;
+#pragma unroll
+                for (int e = 0; e < E; ++e) store_out(out, bf16, (qrow0 + g) * D + lane * E + e, o[g][e] * inv);
+            }
+        }
+    }
+
+    __device__ __forceinline__ void store_partial(float *po, int G) const
+    {
+#pragma unroll
+        for (int g = 0; g < GT; ++g)
+            if (g < G) {
+                float *dst = po + (size_t)g * D + lane * E;
+                if constexpr (E == 4) *reinterpret_cast<float4 *>(dst) = make_float4(o[g][0], o[g][1], o[g][2], o[g][3]);
+                else *reinterpret_cast<float2 *>(dst) = make_float2(o[g][0], o[g][1]);
+            }
+    }
+};
+
+template <class Block>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
-    decode_tma(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a)
+    decode_stream(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a)
 {
-    using LY = TmaLayout<D>;
-    constexpr int NW = kDecodeWarps, S = kDecodeStages, HALVES = LY::HALVES, TILE = LY::TILE;
+    constexpr int D = Block::D, HS = Block::HS, KB = Block::KB, GM = Block::GM;
+    using LY = RingLayout<D>;
+    constexpr int NW = kDecodeWarps, S = kDecodeStages;
     constexpr int STAGE = LY::STAGE;
-    constexpr int MT = D / 16;  // m-tiles of PV (d on M)
+    constexpr int APP = Block::APP;  // 16-byte chunks of the appended K and V rows per lane
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bars[NW * S];  // ring stages of all warps (either partition)
     __shared__ int sm_scan[NW];
     __shared__ int sm_red[2 * NW];  // per warp: most blocks of a unit, units with keys
+    __shared__ __align__(16) float sm_block[Block::SCRATCH > 0 ? NW * Block::SCRATCH : 1];  // the block consumer's
     const uint32_t raw0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
     const uint32_t ring0 = (raw0 + 1023u) & ~1023u;
     int *sm_pre = reinterpret_cast<int *>(smem_raw + (ring0 - raw0) + LY::RING);  // [units + 1]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int units = a.units;
-    if (tid == 0) {  // fetch both tensor-map descriptors (kernel parameters) while the previous kernel drains
+    if (Block::TENSOR_MAPS && tid == 0) {  // fetch both descriptors (kernel parameters) while the previous kernel drains
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
     }
@@ -320,7 +796,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     const long long rs = ring_row(a);  // the ring row this launch writes (-1: none)
 
     // ---- plan: identical in every CTA (lens are not modified until every warp is done).
-    // Each unit's keys form nb_u = ceil(le_u / 16) blocks; the blocks of all units are laid
+    // Each unit's keys form nb_u = ceil(le_u / KB) blocks; the blocks of all units are laid
     // end to end (prefix pb) and every working warp takes one contiguous range of equal
     // length, cut across unit boundaries (a stream-K split).  A unit cut between warps
     // leaves partial (max, sum, output) triples that its last piece merges.  Short units
@@ -365,7 +841,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     {
         int my_b = 0, my_max = 0, my_ne = 0;
         for (int u = u_lo; u < u_hi; ++u) {
-            const int nb = (len_sm[u] + 15) >> 4;
+            const int nb = (len_sm[u] + KB - 1) / KB;
             my_b += nb;
             my_max = max(my_max, nb);
             my_ne += nb > 0;
@@ -388,7 +864,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         for (int w2 = 0; w2 < wid; ++w2) rb += sm_scan[w2];
         for (int u = u_lo; u < u_hi; ++u) {
             pb[u] = rb;
-            rb += (len_sm[u] + 15) >> 4;
+            rb += (len_sm[u] + KB - 1) / KB;
         }
         if (tid == blockDim.x - 1) pb[units] = rb;
     }
@@ -402,8 +878,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // Fewer than half as many units as warps (with at least 8 blocks per warp) also
     // takes the deep partition: there the 8-warp split would cut every unit into many
     // pieces, whose merges cost more than the shallower rings save.
-    const bool deep =
-        NB >= kDeepBlocksPerWarp * total_warps || (NB >= 8 * total_warps && total_warps > 2 * units);
+    const bool deep = Block::DEEP && (NB >= kDeepBlocksPerWarp * total_warps ||
+                                      (NB >= 8 * total_warps && total_warps > 2 * units));
     int max_nb = 0, n_ne = 0;  // most blocks of one unit; units with keys
 #pragma unroll
     for (int w2 = 0; w2 < NW; ++w2) {
@@ -423,7 +899,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         constexpr int NBK = kMaxWholeBlocks + 1;  // buckets: 16 - blocks, so most blocks first
         int *cnt = len_sm + ((units + 31) & ~31);  // [NBK][blockDim.x], also in the idle ring
         for (int k = 0; k < NBK; ++k) cnt[k * blockDim.x + tid] = 0;
-        for (int u = u_lo; u < u_hi; ++u) ++cnt[(kMaxWholeBlocks - ((len_sm[u] + 15) >> 4)) * blockDim.x + tid];
+        for (int u = u_lo; u < u_hi; ++u) ++cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid];
         __syncthreads();
         // exclusive scan of cnt in memory order (bucket-major, then thread): thread t takes
         // entries [NBK t, NBK (t + 1))
@@ -447,7 +923,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         }
         __syncthreads();
         // each thread places its own units, in index order, from its own column of cnt
-        for (int u = u_lo; u < u_hi; ++u) order[cnt[(kMaxWholeBlocks - ((len_sm[u] + 15) >> 4)) * blockDim.x + tid]++] = u;
+        for (int u = u_lo; u < u_hi; ++u) order[cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid]++] = u;
         __syncthreads();
     }
     bool aborted = false;
@@ -456,7 +932,6 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     const uint32_t my_ring = ring0 + (uint32_t)wid * Sm * STAGE;
     // working warps: every one gets at least kMinBlocksPerWarp blocks (or all warps work)
     const int W = max(1, min(NWm * (int)gridDim.x, NB / kMinBlocksPerWarp));
-    const int g = lane >> 2, c = lane & 3;
     const bool out_bf16 = a.out_bf16 != 0;
     auto wstart = [&](int w) { return (int)((long long)w * NB / W); };  // ideal first block of warp w
     auto owner = [&](int b) { return (int)(((long long)(b + 1) * W - 1) / NB); };  // ideal owner of block b
@@ -507,7 +982,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
                 it.Lapp = (le_raw >= 0 && a.append) ? it.le - 1 : -1;
                 it.k0 = 0;
                 it.k1 = it.le;
-                it.nblk = (it.le + 15) >> 4;
+                it.nblk = (it.le + KB - 1) / KB;
                 it.wf = gw;
                 it.nsplit = 1;
                 it.slot = it.slot0 = 0;
@@ -544,8 +1019,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
             it.ub = ub;
             it.le = le_raw >= 0 ? le_raw : 0;
             it.Lapp = (le_raw >= 0 && a.append) ? it.le - 1 : -1;
-            it.k0 = (b_next - ub) * 16;
-            it.k1 = min((bend - ub) * 16, it.le);
+            it.k0 = (b_next - ub) * KB;
+            it.k1 = min((bend - ub) * KB, it.le);
             it.nblk = bend - b_next;
             if (ue - ub <= kMaxWholeBlocks) {  // a short unit: always whole
                 it.wf = gw;
@@ -583,25 +1058,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         return it;
     };
 
-    // Q fragments of an item (rows g < G), head dim permuted to match the K chunks:
-    // k-step j = 4*hh + 2*e + half takes elements 64*hh + 16c + 8e + 4*half + {0,1} (a0)
-    // and + {2,3} (a2).
-    auto load_q = [&](const Item &it, uint32_t (&qa)[D / 16][2]) {
+    Block blk(lane, Block::SCRATCH > 0 ? sm_block + wid * Block::SCRATCH : nullptr);
+    auto load_q = [&](const Item &it) {
         const long qrow = (long)(it.pu / a.Hkv) * a.Hq + (long)(it.pu % a.Hkv) * a.G + it.hp * GS;
-        const int nh = min(GS, a.G - it.hp * GS);
-        const __nv_bfloat16 *qp = reinterpret_cast<const __nv_bfloat16 *>(a.q) + (qrow + g) * D;
-#pragma unroll
-        for (int hh = 0; hh < HALVES; ++hh)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                uint4 wv = make_uint4(0, 0, 0, 0);
-                if (g < nh) wv = *reinterpret_cast<const uint4 *>(qp + 64 * hh + 16 * c + 8 * e);
-                const int j = 4 * hh + 2 * e;
-                qa[j][0] = wv.x;
-                qa[j][1] = wv.y;
-                qa[j + 1][0] = wv.z;
-                qa[j + 1][1] = wv.w;
-            }
+        blk.load_q(a.q, qrow, min(GS, a.G - it.hp * GS));
     };
 
     // K and V rows are read once per launch: evict them first, so they do not displace the
@@ -634,14 +1094,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         if (lane == 0) {
             const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&bars[wid * Sm + slot]);
             const uint32_t dst = my_ring + slot * STAGE;
-            const int y = pit.pu * a.L_cap + pit.k0 + 16 * pblk;
             fence_async_shared();
-            mbar_expect_tx(bar, STAGE);
-#pragma unroll
-            for (int hh = 0; hh < HALVES; ++hh) {
-                tma_load_2d_hint(dst + hh * TILE, &tmK, 64 * hh, y, bar, kv_policy);
-                tma_load_2d_hint(dst + (HALVES + hh) * TILE, &tmV, 64 * hh, y, bar, kv_policy);
-            }
+            const int k = pit.k0 + KB * pblk;  // first key; the appended row is not in the cache yet
+            Block::load(dst, bar, &tmK, &tmV, a, pit.pu, k, min(KB, (pit.Lapp >= 0 ? pit.Lapp : pit.le) - k), kv_policy);
         }
         ++pblk;
         ++issued;
@@ -651,14 +1106,13 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // reads a length from global memory)
     __syncwarp();
     while (issued < (uint32_t)Sm && pblk < pit.nblk) issue();
-    uint32_t qa_n[D / 16][2];  // query fragments of the next item to start
-    if (cur.nblk >= 0) load_q(cur, qa_n);
+    if (cur.nblk >= 0) load_q(cur);  // the queries of the next item to start
     nxt = cur.nblk >= 0 ? next_item() : cur;
     // the launch's queries into the window ring (row rs of every query head's `slots`
     // rows): each warp copies an equal share of 16-byte chunks while its first copies
     // are in flight
     if (a.qring != nullptr && rs >= 0) {
-        constexpr int CH = D / 8;  // 16-byte chunks of a bf16 query row
+        constexpr int CH = Block::ROW / 16;  // 16-byte chunks of a query row
         const long long n16 = a.nq_rows * CH;
         const int tw = (int)gridDim.x * NW, me = (int)blockIdx.x * NW + wid;
         const long long per = (n16 + tw - 1) / tw;
@@ -687,33 +1141,25 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         const long lb = pu / a.Hkv;
         const int h = pu % a.Hkv;
         const int G = min(GS, a.G - cur.hp * GS);
-        const __nv_bfloat16 *kn = a.append ? reinterpret_cast<const __nv_bfloat16 *>(a.k_new) + (long)pu * D : nullptr;
-        const __nv_bfloat16 *vn = a.append ? reinterpret_cast<const __nv_bfloat16 *>(a.v_new) + (long)pu * D : nullptr;
         const long qrow0 = lb * a.Hq + (long)h * a.G + cur.hp * GS;
-        const int row0 = pu * a.L_cap;  // first tensor-map row of this unit
-        // this lane's 16-byte chunk of the appended row (K for lanes < D/8, V for the next
-        // D/8), loaded now so that neither the stage patch nor the cache write below waits
-        // on global memory
-        uint4 app = make_uint4(0, 0, 0, 0);
-        if (Lapp >= k0 && Lapp < k1 && lane < 2 * (D / 8)) {
-            const bool isv = lane >= D / 8;
-            app = *reinterpret_cast<const uint4 *>((isv ? vn : kn) + (isv ? lane - D / 8 : lane) * 8);
+        // this lane's 16-byte chunks of the appended rows (K's chunks, then V's), loaded now so that
+        // neither the stage patch nor the cache write below waits on global memory
+        constexpr int CPR = Block::ROW / 16;
+        uint4 app[APP];
+        const bool has_app = Lapp >= k0 && Lapp < k1;
+#pragma unroll
+        for (int i = 0; i < APP; ++i) {
+            const int p = lane + 32 * i;
+            app[i] = make_uint4(0, 0, 0, 0);
+            if (has_app && p < 2 * CPR)
+                app[i] = reinterpret_cast<const uint4 *>(p < CPR ? a.k_new : a.v_new)[(long)pu * CPR + p % CPR];
         }
 
         // start this item's copies before the wait on its query registers below
         __syncwarp();
         while (issued - consumed < (uint32_t)Sm && can_issue()) issue();
-        uint32_t qa[D / 16][2];
-#pragma unroll
-        for (int j = 0; j < D / 16; ++j) {
-            qa[j][0] = qa_n[j][0];
-            qa[j][1] = qa_n[j][1];
-        }
-        if (nxt.nblk >= 0) load_q(nxt, qa_n);  // the next item's queries load while this one streams
-        float o[MT][4];
-#pragma unroll
-        for (int t = 0; t < MT; ++t) o[t][0] = o[t][1] = o[t][2] = o[t][3] = 0.f;
-        float m = -INFINITY, l = 0.f;
+        blk.start();
+        if (nxt.nblk >= 0) load_q(nxt);  // the next item's queries load while this one streams
 
         for (int bi = 0; bi < cur.nblk; ++bi) {
             __syncwarp();
@@ -728,99 +1174,24 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
                 aborted = true;
                 break;
             }
-            const int kb = k0 + 16 * bi;
-            const uint32_t Ks = my_ring + slot * STAGE, Vs = Ks + HALVES * TILE;
+            const int kb = k0 + KB * bi;
+            const uint32_t Ks = my_ring + slot * STAGE, Vs = Ks + STAGE / 2;
             // patch the stage: zero V rows past the item (K rows there are masked), and
             // put the appended row (not yet in the cache) in place
-            if (kb + 16 > k1 || (Lapp >= kb && Lapp < kb + 16)) {
+            if (kb + KB > k1 || (Lapp >= kb && Lapp < kb + KB)) {
                 const int zr = max(k1 - kb, 0);
-                for (int p = lane; p < (16 - zr) * HALVES * 8; p += 32) {
-                    const int rr = zr + p / (HALVES * 8), ch = p % (HALVES * 8);
-                    sts_u4(Vs + (ch >> 3) * TILE + swz(rr, ch & 7), make_uint4(0, 0, 0, 0));
-                }
-                if (Lapp >= kb && Lapp < kb + 16 && lane < 2 * HALVES * 8) {
-                    const int rr = Lapp - kb;
-                    const bool isv = lane >= HALVES * 8;
-                    const int ch = isv ? lane - HALVES * 8 : lane;
-                    sts_u4((isv ? Vs : Ks) + (ch >> 3) * TILE + swz(rr, ch & 7), app);
+                for (int p = lane; p < (KB - zr) * CPR; p += 32)
+                    sts_u4(Vs + Block::chunk(zr + p / CPR, p % CPR), make_uint4(0, 0, 0, 0));
+                if (Lapp >= kb && Lapp < kb + KB) {
+#pragma unroll
+                    for (int i = 0; i < APP; ++i) {
+                        const int p = lane + 32 * i;
+                        if (p < 2 * CPR) sts_u4((p < CPR ? Ks : Vs) + Block::chunk(Lapp - kb, p % CPR), app[i]);
+                    }
                 }
                 __syncwarp();
             }
-            // four accumulators (keys 0-7 / 8-15, even / odd k-steps): dependent MMA chains
-            // of D/32 instead of D/16
-            float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-            float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int hh = 0; hh < HALVES; ++hh)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const uint4 ka = lds_u4(Ks + hh * TILE + swz(g, 2 * c + e));
-                    const uint4 kc = lds_u4(Ks + hh * TILE + swz(8 + g, 2 * c + e));
-                    const int j = 4 * hh + 2 * e;
-                    mma_bf16(s0, qa[j][0], 0u, qa[j][1], 0u, ka.x, ka.y);
-                    mma_bf16(s1, qa[j][0], 0u, qa[j][1], 0u, kc.x, kc.y);
-                    mma_bf16(t0, qa[j + 1][0], 0u, qa[j + 1][1], 0u, ka.z, ka.w);
-                    mma_bf16(t1, qa[j + 1][0], 0u, qa[j + 1][1], 0u, kc.z, kc.w);
-                }
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                s0[i] += t0[i];
-                s1[i] += t1[i];
-            }
-            // scores of query g for keys kb+2c, kb+2c+1, kb+8+2c, kb+9+2c
-            const int kA = kb + 2 * c, kB = kb + 8 + 2 * c;
-            const float x0 = (kA < k1) ? s0[0] * a.c2 : -INFINITY;
-            const float x1 = (kA + 1 < k1) ? s0[1] * a.c2 : -INFINITY;
-            const float x2 = (kB < k1) ? s1[0] * a.c2 : -INFINITY;
-            const float x3 = (kB + 1 < k1) ? s1[1] * a.c2 : -INFINITY;
-            float mb = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3));
-            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 1));
-            mb = fmaxf(mb, __shfl_xor_sync(0xffffffffu, mb, 2));
-            // Lazy rescale: a row's reference max m moves only when a block max exceeds it
-            // by more than 2^kLazyLog2, so probabilities against a stale m stay <= 2^8
-            // (exact in fp32, and the bf16 hi + lo split keeps 16 bits of them); the
-            // output rescale below then runs on few blocks.  m, l and o stay consistent, so
-            // o / l and lse = m + log2 l are the same quantities as with an exact max.
-            const bool grow = mb > m + kLazyLog2;
-            if (__any_sync(0xffffffffu, grow)) {
-                const float mn = grow ? mb : m;
-                const float alpha = grow ? fast_exp2(m - mn) : 1.f;  // m = -inf gives 0
-                l *= alpha;
-                m = mn;
-                const float a0 = __shfl_sync(0xffffffffu, alpha, (2 * c) * 4);
-                const float a1 = __shfl_sync(0xffffffffu, alpha, (2 * c + 1) * 4);
-#pragma unroll
-                for (int t = 0; t < MT; ++t) {
-                    o[t][0] *= a0;
-                    o[t][1] *= a1;
-                    o[t][2] *= a0;
-                    o[t][3] *= a1;
-                }
-            }
-            const float base = (m == -INFINITY) ? 0.f : m;
-            const float p0 = fast_exp2(x0 - base), p1 = fast_exp2(x1 - base);
-            const float p2 = fast_exp2(x2 - base), p3 = fast_exp2(x3 - base);
-            l += (p0 + p1) + (p2 + p3);
-            // P enters the PV product as bf16 hi + lo parts (two MMAs), which keeps about
-            // 16 significant bits of each probability instead of 8.
-            uint32_t ph0, ph1, pl0, pl1;
-            split_bf16(p0, p1, ph0, pl0);
-            split_bf16(p2, p3, ph1, pl1);
-#pragma unroll
-            for (int hh = 0; hh < HALVES; ++hh) {
-                const uint4 v0 = lds_u4(Vs + hh * TILE + swz(2 * c, g));
-                const uint4 v1 = lds_u4(Vs + hh * TILE + swz(2 * c + 1, g));
-                const uint4 v2 = lds_u4(Vs + hh * TILE + swz(2 * c + 8, g));
-                const uint4 v3 = lds_u4(Vs + hh * TILE + swz(2 * c + 9, g));
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const uint32_t W0 = word(v0, x), W1 = word(v1, x), W2 = word(v2, x), W3 = word(v3, x);
-                    const uint32_t A0 = __byte_perm(W0, W1, 0x5410), A1 = __byte_perm(W0, W1, 0x7632);
-                    const uint32_t A2 = __byte_perm(W2, W3, 0x5410), A3 = __byte_perm(W2, W3, 0x7632);
-                    mma_bf16(o[4 * hh + x], A0, A1, A2, A3, ph0, ph1);
-                    mma_bf16(o[4 * hh + x], A0, A1, A2, A3, pl0, pl1);
-                }
-            }
+            blk.consume(Ks, Vs, kb, k1, a.c2);
             ++consumed;
             if (++c_slot == (uint32_t)Sm) {
                 c_slot = 0;
@@ -829,57 +1200,28 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         }
         if (aborted) break;
 
-        l += __shfl_xor_sync(0xffffffffu, l, 1);
-        l += __shfl_xor_sync(0xffffffffu, l, 2);
+        blk.finish();
 
         // the warp that covers the appended index writes the new row into the cache
-        if (Lapp >= k0 && Lapp < k1 && lane < 2 * (D / 8) && cur.hp == 0) {
-            const bool isv = lane >= D / 8;
-            const int pc = isv ? lane - D / 8 : lane;
-            __nv_bfloat16 *dst = reinterpret_cast<__nv_bfloat16 *>(isv ? a.V : a.K) + ((long)row0 + Lapp) * D + pc * 8;
-            *reinterpret_cast<uint4 *>(dst) = app;
+        if (has_app && cur.hp == 0) {
+#pragma unroll
+            for (int i = 0; i < APP; ++i) {
+                const int p = lane + 32 * i;
+                if (p < 2 * CPR)
+                    reinterpret_cast<uint4 *>(p < CPR ? a.K : a.V)[((long)pu * a.L_cap + Lapp) * CPR + p % CPR] = app[i];
+            }
         }
 
-        const int q0 = 2 * c, q1 = 2 * c + 1;
-        const float l0 = __shfl_sync(0xffffffffu, l, q0 * 4), l1 = __shfl_sync(0xffffffffu, l, q1 * 4);
         if (nsplit == 1) {
-            const float inv0 = l0 > 0.f ? 1.f / l0 : 0.f, inv1 = l1 > 0.f ? 1.f / l1 : 0.f;
-#pragma unroll
-            for (int hh = 0; hh < HALVES; ++hh) {
-                const long d0 = 64 * hh + 8 * g;
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    if (q0 < G) {
-                        store_out<__nv_bfloat16>(a.out, out_bf16, (qrow0 + q0) * D + d0 + 2 * x, o[4 * hh + x][0] * inv0);
-                        store_out<__nv_bfloat16>(a.out, out_bf16, (qrow0 + q0) * D + d0 + 2 * x + 1, o[4 * hh + x][2] * inv0);
-                    }
-                    if (q1 < G) {
-                        store_out<__nv_bfloat16>(a.out, out_bf16, (qrow0 + q1) * D + d0 + 2 * x, o[4 * hh + x][1] * inv1);
-                        store_out<__nv_bfloat16>(a.out, out_bf16, (qrow0 + q1) * D + d0 + 2 * x + 1, o[4 * hh + x][3] * inv1);
-                    }
-                }
-            }
-            if (c == 0 && g < G) put_lse(a, rs, qrow0 + g, l > 0.f ? (m + log2f(l)) * kLn2 : -INFINITY);
+            blk.store(a.out, out_bf16, qrow0, G);
+            blk.each_lse(G, [&](int q, float m, float l) {
+                put_lse(a, rs, qrow0 + q, l > 0.f ? (m + log2f(l)) * kLn2 : -INFINITY);
+            });
         } else {
-            float *po = a.part_o + (size_t)item * GS * D;
-#pragma unroll
-            for (int hh = 0; hh < HALVES; ++hh) {
-                const int d0 = 64 * hh + 8 * g;
-                if (q0 < G) {
-                    float4 *dst = reinterpret_cast<float4 *>(po + (size_t)q0 * D + d0);
-                    dst[0] = make_float4(o[4 * hh + 0][0], o[4 * hh + 0][2], o[4 * hh + 1][0], o[4 * hh + 1][2]);
-                    dst[1] = make_float4(o[4 * hh + 2][0], o[4 * hh + 2][2], o[4 * hh + 3][0], o[4 * hh + 3][2]);
-                }
-                if (q1 < G) {
-                    float4 *dst = reinterpret_cast<float4 *>(po + (size_t)q1 * D + d0);
-                    dst[0] = make_float4(o[4 * hh + 0][1], o[4 * hh + 0][3], o[4 * hh + 1][1], o[4 * hh + 1][3]);
-                    dst[1] = make_float4(o[4 * hh + 2][1], o[4 * hh + 2][3], o[4 * hh + 3][1], o[4 * hh + 3][3]);
-                }
-            }
-            if (c == 0 && g < G) {
-                a.part_ml[((size_t)item * GS + g) * 2 + 0] = m;
-                a.part_ml[((size_t)item * GS + g) * 2 + 1] = l;
-            }
+            blk.store_partial(a.part_o + (size_t)item * GS * D, G);
+            blk.each_lse(G, [&](int q, float m, float l) {
+                reinterpret_cast<float2 *>(a.part_ml)[(size_t)item * GS + q] = make_float2(m, l);
+            });
             // publish: the warp barrier orders every lane's partial writes before lane 0's
             // release; the last arriver's acquire (and the barrier after it) orders its reads
             __syncwarp();
@@ -890,26 +1232,26 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
             if (old == nsplit - 1) {  // last item of this unit: merge the partials
                 if (lane == 0) a.counters[2 + u] = 0;  // every piece has counted: clear for the next launch
                 // pass 1: per-query-head maxima, lanes over splits (independent loads)
-                float Mq[8];
+                float Mq[GM];
 #pragma unroll
-                for (int qq = 0; qq < 8; ++qq) Mq[qq] = -INFINITY;
+                for (int qq = 0; qq < GM; ++qq) Mq[qq] = -INFINITY;
                 for (int sb = 0; sb < nsplit; sb += 32) {
                     const int s2 = sb + lane;
                     if (s2 < nsplit) {
 #pragma unroll
-                        for (int qq = 0; qq < 8; ++qq)
+                        for (int qq = 0; qq < GM; ++qq)
                             if (qq < G)
                                 Mq[qq] = fmaxf(Mq[qq], __ldcg(a.part_ml + ((size_t)(s2 ? 2 * (wf + s2) : slot0) * GS + qq) * 2));
                     }
                 }
 #pragma unroll
-                for (int qq = 0; qq < 8; ++qq) Mq[qq] = warp_max(Mq[qq]);
+                for (int qq = 0; qq < GM; ++qq) Mq[qq] = warp_max(Mq[qq]);
                 // pass 2: every lane owns 4 head-dim elements of all G heads; one sweep over
                 // the splits with all of a split's loads issued together
                 constexpr int PER = D / 32;
-                float acc[8][PER], Lq[8];
+                float acc[GM][PER], Lq[GM];
 #pragma unroll
-                for (int qq = 0; qq < 8; ++qq) {
+                for (int qq = 0; qq < GM; ++qq) {
                     Lq[qq] = 0.f;
 #pragma unroll
                     for (int e = 0; e < PER; ++e) acc[qq][e] = 0.f;
@@ -918,7 +1260,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
                 for (int s2 = 0; s2 < nsplit; ++s2) {
                     const size_t it0 = (size_t)(s2 ? 2 * (wf + s2) : slot0) * GS;
 #pragma unroll
-                    for (int qq = 0; qq < 8; ++qq) {
+                    for (int qq = 0; qq < GM; ++qq) {
                         if (qq < G && Mq[qq] != -INFINITY) {
                             const float2 ml = __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + it0 + qq);
                             const float wt = fast_exp2(ml.x - Mq[qq]);
@@ -938,12 +1280,12 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
                     }
                 }
 #pragma unroll
-                for (int qq = 0; qq < 8; ++qq) {
+                for (int qq = 0; qq < GM; ++qq) {
                     if (qq < G) {
                         const float inv = Lq[qq] > 0.f ? 1.f / Lq[qq] : 0.f;
 #pragma unroll
                         for (int e = 0; e < PER; ++e)
-                            store_out<__nv_bfloat16>(a.out, out_bf16, (qrow0 + qq) * D + lane * PER + e,
+                            store_out(a.out, out_bf16, (qrow0 + qq) * D + lane * PER + e,
                                                      acc[qq][e] * inv);
                         if (lane == 0)
                             put_lse(a, rs, qrow0 + qq, Lq[qq] > 0.f ? (Mq[qq] + log2f(Lq[qq])) * kLn2 : -INFINITY);
@@ -1056,6 +1398,20 @@ static bool encode_cache_map(CUtensorMap *map, const void *base, unsigned long l
     return encode_bf16_2d(map, base, rows, d, 64, 16);
 }
 
+typedef void (*DecodeKernel)(CUtensorMap, CUtensorMap, DecodeArgs);
+
+// float32 kernel for up to gt (2, 4, 6 or 8) query heads per virtual unit, hs of them per unit.
+template <int D> static DecodeKernel f32_kernel(int gt, int hs)
+{
+    if (hs == 2) return decode_stream<F32Block<D, 8, 2>>;
+    switch (gt) {
+    case 2: return decode_stream<F32Block<D, 2, 1>>;
+    case 4: return decode_stream<F32Block<D, 4, 1>>;
+    case 6: return decode_stream<F32Block<D, 6, 1>>;
+    default: return decode_stream<F32Block<D, 8, 1>>;
+    }
+}
+
 cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, const void *v_new,
                           int32_t *lens, float scale, void *out, reco_dtype out_dtype, float *lse,
                           const DecodeWs &ws, unsigned *err, cudaStream_t s, float *ring, int slots,
@@ -1087,39 +1443,41 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
     a.slots = slots;
     a.nq = (long long)kv.n_layers * kv.B * kv.H_q;
     a.qring = ring ? qring : nullptr;
-    a.q_bytes = kv.dtype == RECO_F32 ? 4 : 2;
     a.nq_rows = a.nq;
     a.advance = 1;
-    // partial slots: two per warp of the grid
-    const bool slots_fit = 2LL * device_sm_count() * kDecodeWarps <= (long long)ws.part_slots;
-    // the TMA path takes up to 8 query heads per unit; a unit of G <= 16 heads is two
-    // virtual units of ceil(G / 2) heads each
-    a.hs = a.G > 8 ? 2 : 1;
-    a.gv = (a.G + a.hs - 1) / a.hs;
+    const bool f32 = kv.dtype == RECO_F32;
+    // query heads per virtual unit: float32 units of more than 8 heads run as two of half as many
+    const int hs = f32 && a.G > 8 ? 2 : 1;
+    a.gv = (a.G + hs - 1) / hs;
+    DecodeKernel fn;
+    if (f32) {
+        const int gt = std::min(8, (a.gv + 1) / 2 * 2);
+        fn = kv.d == 64 ? f32_kernel<64>(gt, hs) : f32_kernel<128>(gt, hs);
+    } else {
+        fn = kv.d == 64 ? (a.G > 8 ? decode_stream<Bf16Block<64, 2>> : decode_stream<Bf16Block<64, 1>>)
+                        : (a.G > 8 ? decode_stream<Bf16Block<128, 2>> : decode_stream<Bf16Block<128, 1>>);
+    }
     // More units than one plan holds in shared memory run as consecutive launches over
     // contiguous unit ranges (every unit is independent): each part gets its own K/V, q,
     // output, lens and ring pointers, and only the last part advances the ring slot.
-    const long long part_units = kMaxTmaUnits / a.hs;  // cache units per launch
-    if (kv.dtype == RECO_BF16 && a.G <= 16 && (unsigned long long)std::min<long long>(a.units, part_units) * kv.L_cap <
-                                                   (1ull << 31) && slots_fit) {
-        const bool two = a.hs == 2;
-        const void *fn = kv.d == 64 ? (two ? (const void *)decode_tma<64, 2> : (const void *)decode_tma<64, 1>)
-                                    : (two ? (const void *)decode_tma<128, 2> : (const void *)decode_tma<128, 1>);
-        const size_t row_b = (size_t)kv.d * 2;  // bf16 cache and query rows
+    const long long part_units = (f32 ? kMaxF32Units : kMaxTmaUnits) / hs;  // cache units per launch
+    // bf16 rows are addressed by tensor-map coordinates
+    if (f32 || (unsigned long long)std::min<long long>(a.units, part_units) * kv.L_cap < (1ull << 31)) {
+        const size_t row_b = (size_t)kv.d * (f32 ? 4 : 2);  // cache and query rows
         const size_t out_b = (size_t)kv.d * (out_dtype == RECO_BF16 ? 2 : 4);
         for (long long u0 = 0; u0 < a.units; u0 += part_units) {
             const long long cu = std::min(part_units, (long long)a.units - u0);
             const long long q0 = u0 * a.G;  // first query head of the part
             const unsigned long long rows = (unsigned long long)cu * kv.L_cap;
-            CUtensorMap mk, mv;
+            CUtensorMap mk = {}, mv = {};
             const char *kb = static_cast<const char *>(kv.k) + (size_t)u0 * kv.L_cap * row_b;
             const char *vb = static_cast<const char *>(kv.v) + (size_t)u0 * kv.L_cap * row_b;
-            if (!encode_cache_map(&mk, kb, rows, kv.d) || !encode_cache_map(&mv, vb, rows, kv.d)) {
+            if (!f32 && (!encode_cache_map(&mk, kb, rows, kv.d) || !encode_cache_map(&mv, vb, rows, kv.d))) {
                 if (u0 == 0) break;  // the SIMT path below takes the whole call
                 return cudaErrorInvalidValue;
             }
             DecodeArgs at = a;  // virtual units of this part
-            at.units = (int)(cu * a.hs);
+            at.units = (int)(cu * hs);
             at.K = const_cast<char *>(kb);
             at.V = const_cast<char *>(vb);
             at.q = static_cast<const char *>(q) + (size_t)q0 * row_b;
@@ -1133,35 +1491,25 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
             at.nq_rows = cu * a.G;
             at.advance = u0 + cu >= a.units ? 1 : 0;
             // the counters are zero on entry (zero-filled workspace) and every launch leaves them so
-            const size_t smem = kv.d == 64 ? tma_smem_bytes<64>(at.units) : tma_smem_bytes<128>(at.units);
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            const size_t smem = kv.d == 64 ? ring_smem_bytes<64>(at.units) : ring_smem_bytes<128>(at.units);
+            cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            const int grid = device_sm_count();
-            const dim3 blk(kDecodeWarps * 32);
-            if (kv.d == 64)
-                e = two ? launch_pdl(decode_tma<64, 2>, dim3(grid), blk, smem, s, mk, mv, at)
-                        : launch_pdl(decode_tma<64, 1>, dim3(grid), blk, smem, s, mk, mv, at);
-            else
-                e = two ? launch_pdl(decode_tma<128, 2>, dim3(grid), blk, smem, s, mk, mv, at)
-                        : launch_pdl(decode_tma<128, 1>, dim3(grid), blk, smem, s, mk, mv, at);
+            // two partial slots per warp of the grid
+            const int grid = std::min(device_sm_count(), ws.part_slots / (2 * kDecodeWarps));
+            e = launch_pdl(fn, dim3(grid), dim3(kDecodeWarps * 32), smem, s, mk, mv, at);
             if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
             if (u0 + cu >= a.units) return cudaSuccess;
         }
     }
-    a.hs = 1;
+    // bf16 caches that no tensor map covers
     a.gv = a.G;
     const unsigned grid = (unsigned)a.units;
-    if (kv.dtype == RECO_F32) {
-        if (kv.d == 64) decode_simt<float, 64><<<grid, 128, 0, s>>>(a);
-        else decode_simt<float, 128><<<grid, 128, 0, s>>>(a);
-    } else {
-        if (kv.d == 64) decode_simt<__nv_bfloat16, 64><<<grid, 128, 0, s>>>(a);
-        else decode_simt<__nv_bfloat16, 128><<<grid, 128, 0, s>>>(a);
-    }
+    if (kv.d == 64) decode_simt<__nv_bfloat16, 64><<<grid, 128, 0, s>>>(a);
+    else decode_simt<__nv_bfloat16, 128><<<grid, 128, 0, s>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || !ring) return e;
     if (a.qring) {
-        const int ch = kv.d * a.q_bytes / 16;
+        const int ch = kv.d * 2 / 16;
         const long long n16 = a.nq * ch;
         const unsigned blocks = (unsigned)std::min<long long>((n16 + 255) / 256, 4LL * device_sm_count());
         qring_copy<<<blocks, 256, 0, s>>>(reinterpret_cast<const uint4 *>(q), reinterpret_cast<uint4 *>(a.qring), n16,
