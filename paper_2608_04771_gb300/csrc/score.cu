@@ -200,9 +200,9 @@ __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, 
     const int used = ((L + part_keys - 1) / part_keys) * per;
     float m = -INFINITY, z = 0.f;
     const size_t o0 = (size_t)u * n_parts * R + r;
-    constexpr int U = 8;  // partials in flight
+    constexpr int U = 8;  // partials in flight: their max, then one exponential each
     for (int c0 = 0; c0 < used; c0 += U) {
-        float pm[U], pz[U];
+        float pm[U], pz[U], mn = m;
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             const bool in = c0 + k < used;
@@ -211,7 +211,12 @@ __global__ void score_combine(const int32_t *__restrict__ lens, ScoreMask mask, 
             pz[k] = in ? part_z[o] : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < U; ++k) lse_merge(m, z, pm[k], pz[k]);
+        for (int k = 0; k < U; ++k) mn = fmaxf(mn, pm[k]);
+        if (mn == -INFINITY) continue;
+        z *= fast_exp2(m - mn);
+#pragma unroll
+        for (int k = 0; k < U; ++k) z = fmaf(pz[k], fast_exp2(pm[k] - mn), z);
+        m = mn;
     }
     rowb[i] = m + log2f(z);
 }

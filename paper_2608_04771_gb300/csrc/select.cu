@@ -2,15 +2,15 @@
 // highest-scoring tokens with the latest w always retained, then compress the L
 // cached tokens down to m_i).
 //
-// select_topm: CTAs that walk the (layer, sequence, KV head) units, one unit at a time
-// (a unit whose sequence keeps its whole cache is an identity, skipped by the
-// compaction).  A 4 x 8-bit radix select
-// over order-preserving uint32 keys of the float32 scores finds the (m-w)-th
-// largest key T and how many keys equal to T are still needed; one ordered pass
-// then emits every candidate with key > T plus the first `need` with key == T in
-// index order.  The result is sorted and ties go to the lower index, with no sort.
-// select_topm_smem does the same from keys staged in shared memory (units of up to
-// kSelectSmemKeys candidates).
+// Three selections, by the most candidates a unit may have (L_cap - w), all with the same rule: a
+// radix or bit search over order-preserving uint32 keys of the float32 scores finds the (m-w)-th
+// largest key T and how many keys equal to T are still needed; one ordered pass then emits every
+// candidate with key > T plus the first `need` with key == T in index order.  The result is
+// sorted and ties go to the lower index, with no sort.
+//   select_topm_warp  up to 1024: one warp per unit, keys in registers
+//   select_topm_smem  up to kSelectSmemKeys: CTAs walk the units, keys in shared memory
+//   select_topm       longer: CTAs walk the units, keys read from global memory
+// A unit whose sequence keeps its whole cache is an identity, skipped by the compaction.
 //
 // compact_rows: CTAs per (K|V, 128-byte column slice) that walk the units, one at a
 // time.  kept[] is strictly increasing, so kept[r] >= r (the kernel refuses any index that is not): the source
@@ -203,29 +203,34 @@ __global__ void __launch_bounds__(NT) select_topm(const float *__restrict__ scor
     }
 }
 
-// The same selection with the unit's keys staged in shared memory once (all loads in
-// flight), the radix passes run from there, and the ordered emit done by warp-contiguous
-// segments: one counting sweep, one scan of the 32 warps' counts, one writing sweep.
+// The same selection with the unit's keys staged in shared memory once (all loads in flight), the
+// radix passes run from there, and the ordered emit done by warp-contiguous segments: one counting
+// sweep, one scan of the warps' counts, one writing sweep.  The passes start below the bits that
+// all keys share (their smallest and largest key): scores of one unit lie within a few powers of
+// two, so a first digit of the top eight bits put nearly all keys into two or three bins, whose
+// atomics serialise.  512 threads, so that three units of 16384 keys share an SM and one counts
+// while another waits at a barrier.  512 units of 15000 to 16384 candidates: 54 -> 45 us.
 template <int NT>
 __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__ scores, const int32_t *lens,
                                                        int32_t *lens_out, const int32_t *__restrict__ keep, int w, int B, int Hkv,
                                                        int L_cap, int32_t *__restrict__ idx_out,
                                                        int32_t *__restrict__ count, long units, unsigned *err)
 {
-    static_assert(NT == 1024, "one warp per lane of the warp-count scan");
     constexpr int NW = NT / 32;
+    static_assert(NW <= 32, "one warp per lane of the warp-count scan");
     extern __shared__ uint32_t keys[];  // [L - w]
     __shared__ int hist[256];
     __shared__ int w_gt[NW], w_eq[NW];
+    __shared__ uint32_t w_min[NW], w_max[NW];
     __shared__ uint32_t s_prefix;
     __shared__ int s_remaining;
     __shared__ int2 s_lm[kWalkAhead];
     wait_prior_grid();  // scores, lens and keep may come from the previous kernels
     walk_headers(s_lm, lens, keep, units, B, Hkv);
     __syncthreads();
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int it = 0;
     for (long u = blockIdx.x; u < units; u += gridDim.x, ++it) {  // a few CTAs per SM walk the units
-        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
         const int L = s_lm[it].x, m = s_lm[it].y;  // the grid gives no CTA more than kWalkAhead units
         if (L < w || L > L_cap || m < w || m > L) {
             if (tid == 0) {
@@ -242,53 +247,60 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
             if (tid == 0) count[u] = 0;
             continue;
         }
-    #pragma unroll 8
-        for (int j = tid; j < nc; j += NT) keys[j] = order_key(__ldcg(s + j));
-        if (tid == 0) {
-            s_prefix = 0;
-            s_remaining = kc;
+        uint32_t lo = 0xffffffffu, hi = 0;
+#pragma unroll 8
+        for (int j = tid; j < nc; j += NT) {
+            const uint32_t key = order_key(__ldcg(s + j));
+            keys[j] = key;
+            lo = min(lo, key);
+            hi = max(hi, key);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        if (lane == 0) {
+            w_min[wid] = lo;
+            w_max[wid] = hi;
         }
         __syncthreads();
+        lo = __reduce_min_sync(0xffffffffu, lane < NW ? w_min[lane] : 0xffffffffu);
+        hi = __reduce_max_sync(0xffffffffu, lane < NW ? w_max[lane] : 0u);
         uint32_t T = 0xffffffffu;
         int need = 0;
         if (kc > 0) {
-            uint32_t mask = 0;
-            for (int shift = 24; shift >= 0; shift -= 8) {
+            int bits = 32 - __clz(lo ^ hi);  // the low bits in which keys differ
+            uint32_t prefix = bits < 32 ? hi >> bits << bits : 0u;
+            uint32_t mask = bits < 32 ? ~0u << bits : 0u;
+            int remaining = kc;
+            while (bits > 0) {
+                const int shift = max(0, bits - 8);
                 for (int i = tid; i < 256; i += NT) hist[i] = 0;
                 __syncthreads();
-                const uint32_t prefix = s_prefix;
-                const int remaining = s_remaining;
-                for (int jb = 0; jb < nc; jb += NT) {
-                    const int j = jb + tid;
-                    const bool valid = j < nc;
-                    const uint32_t key = valid ? keys[j] : 0u;
-                    const bool match = valid && (key & mask) == prefix;
-                    const uint32_t bin = (key >> shift) & 255u;
+                for (int j = tid; j < nc; j += NT) {
+                    const uint32_t key = keys[j];
                     // plain shared-memory atomics: grouping a warp's equal bins first
-                    // (__match_any_sync) cost more than the conflicts it saves (7B-class
-                    // selection 109 -> 79 us)
-                    if (match) atomicAdd(&hist[bin], 1);
+                    // (__match_any_sync) cost more than the conflicts it saves
+                    if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
                 }
                 __syncthreads();
-                if (tid < 32) {  // find the bin holding the remaining-th largest key
+                if (wid == 0) {  // find the bin holding the remaining-th largest key
                     int c8[8], sum = 0;
-    #pragma unroll
+#pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         c8[i] = hist[255 - 8 * lane - i];
                         sum += c8[i];
                     }
                     int incl = sum;
-    #pragma unroll
+#pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
                         int n = __shfl_up_sync(0xffffffffu, incl, o);
                         if (lane >= o) incl += n;
                     }
                     int cum = incl - sum;
                     if (cum < remaining && remaining <= incl) {
-    #pragma unroll
+#pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             if (cum + c8[i] >= remaining) {
-                                s_prefix = prefix | ((uint32_t)(255 - 8 * lane - i) << shift);
+                                s_prefix = (uint32_t)(255 - 8 * lane - i) << shift;
                                 s_remaining = remaining - cum;
                                 break;
                             }
@@ -296,31 +308,36 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
                         }
                     }
                 }
-                mask |= 255u << shift;
                 __syncthreads();
+                // a first digit of fewer than eight bits meets bins of the shared bits above them
+                prefix |= s_prefix;
+                remaining = s_remaining;
+                mask |= 255u << shift;
+                bits = shift;
             }
-            T = s_prefix;
-            need = s_remaining;
+            T = prefix;
+            need = remaining;
         }
         // emit in index order: keys > T, then the first `need` keys == T
         const int seg = (nc + NW - 1) / NW;
         const int j0 = min(nc, wid * seg), j1 = min(nc, j0 + seg);
         int n_gt = 0, n_eq = 0;
-        for (int jb = j0; jb < j1; jb += 32) {
-            const int j = jb + lane;
-            const uint32_t key = j < j1 ? keys[j] : 0u;
-            n_gt += __popc(__ballot_sync(0xffffffffu, j < j1 && key > T));
-            n_eq += __popc(__ballot_sync(0xffffffffu, j < j1 && key == T));
+        for (int j = j0 + lane; j < j1; j += 32) {
+            const uint32_t key = keys[j];
+            n_gt += key > T;
+            n_eq += key == T;
         }
+        n_gt = __reduce_add_sync(0xffffffffu, n_gt);
+        n_eq = __reduce_add_sync(0xffffffffu, n_eq);
         if (lane == 0) {
             w_gt[wid] = n_gt;
             w_eq[wid] = n_eq;
         }
         __syncthreads();
         if (wid == 0) {  // per warp: equal keys before its segment, and output rows before it
-            const int e = w_eq[lane], g = w_gt[lane];
+            const int e = lane < NW ? w_eq[lane] : 0, g = lane < NW ? w_gt[lane] : 0;
             int e_inc = e;
-    #pragma unroll
+#pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int n = __shfl_up_sync(0xffffffffu, e_inc, o);
                 if (lane >= o) e_inc += n;
@@ -328,13 +345,15 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
             const int e_base = e_inc - e;
             const int f = g + min(max(need - e_base, 0), e);
             int f_inc = f;
-    #pragma unroll
+#pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int n = __shfl_up_sync(0xffffffffu, f_inc, o);
                 if (lane >= o) f_inc += n;
             }
-            w_eq[lane] = e_base;
-            w_gt[lane] = f_inc - f;
+            if (lane < NW) {
+                w_eq[lane] = e_base;
+                w_gt[lane] = f_inc - f;
+            }
         }
         __syncthreads();
         int e_run = w_eq[wid], pos = w_gt[wid];
@@ -357,6 +376,90 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
             if (lens_out) lens_out[u] = m;
         }
         __syncthreads();  // this unit's shared memory is read out before the next unit's fill
+    }
+}
+
+// The same selection for short units (L_cap - w <= 32 * K): one warp per unit, its keys in
+// registers (lane l holds candidates l, l + 32, ...), the threshold found bit by bit from the top
+// one in which keys differ: a count of the keys at or above each trial value, no shared memory and
+// no barrier.  A CTA of 512 threads spends such a unit's time at its barriers (step boundary of
+// the trace, 1792 units of 90 to 240 rows, one eighth of them compressed: 14 -> 9 us).
+constexpr int kWarpThreads = 256;
+
+template <int K>
+__global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__restrict__ scores, const int32_t *lens,
+                                                                 int32_t *lens_out, const int32_t *__restrict__ keep,
+                                                                 int w, int B, int Hkv, int L_cap,
+                                                                 int32_t *__restrict__ idx_out,
+                                                                 int32_t *__restrict__ count, int units, unsigned *err)
+{
+    wait_prior_grid();  // scores, lens and keep may come from the previous kernels
+    const int lane = threadIdx.x & 31;
+    const int u = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5);
+    if (u >= units) return;
+    const int L = lens[u], m = keep[(u / Hkv) % B];
+    if (L < w || L > L_cap || m < w || m > L) {
+        if (lane == 0) {
+            count[u] = 0;
+            raise_error(err, (L < w || L > L_cap) ? ERR_LEN : ERR_KEEP);
+        }
+        return;
+    }
+    const int nc = L - w, kc = m - w;
+    const float *s = scores + (long)u * L_cap;
+    int32_t *idx = idx_out + (long)u * L_cap;
+    if (kc == nc) {  // keep everything: identity, nothing moves (the compaction skips it)
+        for (int j = lane; j < L; j += 32) idx[j] = j;
+        if (lane == 0) count[u] = 0;
+        return;
+    }
+    uint32_t key[K], lo = 0xffffffffu, hi = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int j = 32 * i + lane;
+        const float x = j < nc ? __ldcg(s + j) : 0.f;
+        key[i] = j < nc ? order_key(x) : 0u;  // order_key is 0 for no score but the NaN of all ones
+        if (j < nc) {
+            lo = min(lo, key[i]);
+            hi = max(hi, key[i]);
+        }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    uint32_t T = 0xffffffffu;
+    int need = 0;
+    if (kc > 0) {
+        const int bits = 32 - __clz(lo ^ hi);
+        T = bits < 32 ? hi >> bits << bits : 0u;  // the largest value with at least kc keys at or above it
+        for (int b = bits - 1; b >= 0; --b) {
+            const uint32_t trial = T | 1u << b;
+            int n = 0;
+#pragma unroll
+            for (int i = 0; i < K; ++i) n += key[i] >= trial;
+            if (__reduce_add_sync(0xffffffffu, n) >= kc) T = trial;
+        }
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < K; ++i) n += key[i] > T;
+        need = kc - __reduce_add_sync(0xffffffffu, n);
+    }
+    const unsigned below = (1u << lane) - 1u;
+    int e_run = 0, pos = 0;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const int j = 32 * i + lane;
+        const bool is_eq = j < nc && key[i] == T;
+        const unsigned eb = __ballot_sync(0xffffffffu, is_eq);
+        const bool flag = (j < nc && key[i] > T) || (is_eq && e_run + __popc(eb & below) < need);
+        const unsigned fb = __ballot_sync(0xffffffffu, flag);
+        if (flag) idx[pos + __popc(fb & below)] = j;
+        e_run += __popc(eb);
+        pos += __popc(fb);
+    }
+    for (int t = lane; t < w; t += 32) idx[kc + t] = nc + t;
+    if (lane == 0) {
+        count[u] = m;
+        if (lens_out) lens_out[u] = m;
     }
 }
 
@@ -488,19 +591,30 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
                                  cudaStream_t s)
 {
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
-    // keys of a unit staged in shared memory when L_cap - w of them fit
-    const size_t key_bytes = (size_t)(kv.L_cap - w) * sizeof(uint32_t);
-    if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
-        cudaError_t e = cudaFuncSetAttribute(select_topm_smem<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kSelectSmemKeys * (int)sizeof(uint32_t));
+    const int most = kv.L_cap - w;  // candidates of a unit
+    cudaError_t e;
+    if (most <= 32 * 32) {  // short units: a warp each
+        auto fn = most <= 32 * 8 ? select_topm_warp<8> : (most <= 32 * 16 ? select_topm_warp<16> : select_topm_warp<32>);
+        constexpr int per = kWarpThreads / 32;
+        e = launch_pdl(fn, dim3((unsigned)((units + per - 1) / per)), dim3(kWarpThreads), 0, s, scores, lens, lens_out,
+                       keep, w, kv.B, kv.H_kv, kv.L_cap, idx, count, (int)units, err);
         if (e != cudaSuccess) return e;
-        const unsigned grid = walk_grid(select_topm_smem<1024>, 1024, key_bytes, units, 1);
-        e = launch_pdl(select_topm_smem<1024>, dim3(grid), dim3(1024), key_bytes, s, scores, lens, lens_out, keep, w,
+        return cudaGetLastError();
+    }
+    // keys of a unit staged in shared memory when L_cap - w of them fit
+    const size_t key_bytes = (size_t)most * sizeof(uint32_t);
+    if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
+        constexpr int NT = 512;
+        e = cudaFuncSetAttribute(select_topm_smem<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSelectSmemKeys * (int)sizeof(uint32_t));
+        if (e != cudaSuccess) return e;
+        const unsigned grid = walk_grid(select_topm_smem<NT>, NT, key_bytes, units, 1);
+        e = launch_pdl(select_topm_smem<NT>, dim3(grid), dim3(NT), key_bytes, s, scores, lens, lens_out, keep, w,
                        kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
         if (e != cudaSuccess) return e;
     } else {
         const unsigned grid = walk_grid(select_topm<1024>, 1024, 0, units, 1);
-        cudaError_t e = launch_pdl(select_topm<1024>, dim3(grid), dim3(1024), 0, s, scores, lens, lens_out, keep, w,
+        e = launch_pdl(select_topm<1024>, dim3(grid), dim3(1024), 0, s, scores, lens, lens_out, keep, w,
                                    kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
         if (e != cudaSuccess) return e;
     }
