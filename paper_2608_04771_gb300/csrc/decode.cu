@@ -783,8 +783,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int units = a.units;
     if (Block::TENSOR_MAPS && tid == 0) {  // fetch both descriptors (kernel parameters) while the previous kernel drains
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmK)) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
+        prefetch_tensormap(&tmK);
+        prefetch_tensormap(&tmV);
     }
     if (lane == 0) {
         for (int s2 = 0; s2 < S; ++s2) mbar_init((uint32_t)__cvta_generic_to_shared(&bars[wid * S + s2]), 1);

@@ -40,7 +40,7 @@ struct ScoreMask {
 #ifdef __CUDACC__
     __device__ __forceinline__ bool skip(long u, int L, int w, int L_cap) const
     {
-        return keep != nullptr && L >= w && L <= L_cap && keep[(u / Hkv) % B] >= L;
+        return keep != nullptr && L >= w && L <= L_cap && keep[((int)u / Hkv) % B] >= L;
     }
 #endif
 };

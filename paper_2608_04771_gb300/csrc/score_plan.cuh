@@ -36,14 +36,16 @@ __device__ __forceinline__ int plan_runs(TilePlan &pl, const int32_t *__restrict
     const int u_lo = min(units, tid * seg), u_hi = min(units, u_lo + seg);
     auto keys_of = [&](int u, int &L) {
         L = lens[u];
+        const int kp = mask.keep != nullptr ? mask.keep[(u / mask.Hkv) % mask.B] : 0;  // (its load does not wait for the length)
         if (L < w || L > L_cap) {
             if (err_len != nullptr && blockIdx.x == 0 && skip == 0) raise_error(err_len, ERR_LEN);
             return 0;
         }
-        if (mask.skip(u, L, w, L_cap)) return 0;
+        if (mask.keep != nullptr && kp >= L) return 0;
         return candidates_only ? L - w : L;
     };
     int my_i = 0, my_n = 0;
+#pragma unroll 4
     for (int u = u_lo; u < u_hi; ++u) {
         int L;
         const int k = keys_of(u, L);

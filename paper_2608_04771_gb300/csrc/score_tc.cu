@@ -276,6 +276,8 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
     const uint32_t Qs = base;              // MT x HALVES x BOX
     const uint32_t Ks = base + C::QBYTES;  // NS x KSTAGE
     if (tid == 0) {
+        prefetch_tensormap(&tmQ);
+        prefetch_tensormap(&tmK);
         mbar_init(smem_addr(&bar_qfull), 1);
         mbar_init(smem_addr(&bar_qempty), 1);
         for (int s = 0; s < NS; ++s) {
@@ -542,6 +544,8 @@ __global__ void __launch_bounds__(64 + 128 * kP2Groups, 1)
     // per epilogue warp: the normalisers of its columns, after the K ring
     float *bsh = reinterpret_cast<float *>(smem_raw + (base - raw0) + HALVES * QBOXB + (size_t)NS * KSTAGE);
     if (tid == 0) {
+        prefetch_tensormap(&tmQ);
+        prefetch_tensormap(&tmK);
         mbar_init(smem_addr(&bar_qfull), 1);
         mbar_init(smem_addr(&bar_qempty), 1);
         for (int s = 0; s < NS; ++s) {

@@ -433,10 +433,10 @@ __global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__
         T = bits < 32 ? hi >> bits << bits : 0u;  // the largest value with at least kc keys at or above it
         for (int b = bits - 1; b >= 0; --b) {
             const uint32_t trial = T | 1u << b;
-            int n = 0;
+            int n[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int i = 0; i < K; ++i) n += key[i] >= trial;
-            if (__reduce_add_sync(0xffffffffu, n) >= kc) T = trial;
+            for (int i = 0; i < K; ++i) n[i & 3] += key[i] >= trial;
+            if (__reduce_add_sync(0xffffffffu, (n[0] + n[1]) + (n[2] + n[3])) >= kc) T = trial;
         }
         int n = 0;
 #pragma unroll
