@@ -103,6 +103,29 @@ int device_sm_count()
     }
     return g_sm_count[dev];
 }
+cudaError_t allow_smem(const void *kernel, int bytes)
+{
+    struct Entry {
+        const void *kernel;
+        int dev, bytes;
+    };
+    constexpr int kMax = 512;
+    static Entry have[kMax];
+    static int n = 0;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_mu);
+    int i = 0;
+    while (i < n && (have[i].kernel != kernel || have[i].dev != dev)) ++i;
+    if (i < n && have[i].bytes >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    if (i == n && n < kMax) have[n++] = Entry{kernel, dev, bytes};
+    else if (i < n) have[i].bytes = bytes;
+    return cudaSuccess;
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);

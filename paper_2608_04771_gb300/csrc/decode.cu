@@ -1492,7 +1492,7 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
             at.advance = u0 + cu >= a.units ? 1 : 0;
             // the counters are zero on entry (zero-filled workspace) and every launch leaves them so
             const size_t smem = kv.d == 64 ? ring_smem_bytes<64>(at.units) : ring_smem_bytes<128>(at.units);
-            cudaError_t e = cudaFuncSetAttribute((const void *)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = allow_smem((const void *)fn, (int)smem);
             if (e != cudaSuccess) return e;
             // two partial slots per warp of the grid
             const int grid = std::min(device_sm_count(), ws.part_slots / (2 * kDecodeWarps));

@@ -529,7 +529,7 @@ static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *
     cudaError_t e = cudaSuccess;
     if (pass1) {
         const int n_parts = score_row_parts(kv, w), part_tiles = simt_part_tiles(kv, w);
-        e = cudaFuncSetAttribute(score_rowstats_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_smem((const void *)score_rowstats_simt<T, D>, (int)smem);
         if (e != cudaSuccess) return e;
         e = launch_pdl(score_rowstats_simt<T, D>, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv,
                        kv.L_cap, R, n_parts, part_tiles, (int)units, c2, ws.part_m, ws.part_z, err);
@@ -539,7 +539,7 @@ static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *
                        units);
         if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(score_colsum_simt<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem((const void *)score_colsum_simt<T, D>, (int)smem);
     if (e != cudaSuccess) return e;
     e = launch_pdl(score_colsum_simt<T, D>, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap,
                    R, (int)units, c2, (const float *)ws.rowb, ws.raw, mask.keep ? ws.ulist : nullptr,

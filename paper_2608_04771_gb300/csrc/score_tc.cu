@@ -791,8 +791,7 @@ static cudaError_t run_pass1(const reco_kv &kv, const void *q_win, const int32_t
         *ok = false;
         return cudaSuccess;
     }
-    cudaError_t e = cudaFuncSetAttribute(score_rowstats_tc<D, MT, EG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)C::SMEM);
+    cudaError_t e = allow_smem((const void *)score_rowstats_tc<D, MT, EG>, (int)C::SMEM);
     if (e != cudaSuccess) return e;
     const int grid = (int)min(units * nch, (long)device_sm_count());
     e = launch_pdl(score_rowstats_tc<D, MT, EG>, dim3(grid), dim3(C::THREADS), C::SMEM, s, mq, mk, lens, mask, w,
@@ -849,7 +848,7 @@ static cudaError_t run_pass2(const reco_kv &kv, const void *q_win, const int32_t
     }
     const int NS = (int)min((size_t)4, (budget - qbytes - nbytes) / kstage);
     const size_t smem = 1024 + qbytes + (size_t)NS * kstage + nbytes;
-    cudaError_t e = cudaFuncSetAttribute(score_colsum_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem((const void *)score_colsum_tc<D>, (int)smem);
     if (e != cudaSuccess) return e;
     const long tiles = units * ((kv.L_cap + kTile - 1) / kTile);
     const int grid = (int)min(tiles, (long)device_sm_count());

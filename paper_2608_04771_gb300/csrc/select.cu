@@ -605,8 +605,7 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
     const size_t key_bytes = (size_t)most * sizeof(uint32_t);
     if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
         constexpr int NT = 512;
-        e = cudaFuncSetAttribute(select_topm_smem<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kSelectSmemKeys * (int)sizeof(uint32_t));
+        e = allow_smem((const void *)select_topm_smem<NT>, (int)kSelectSmemKeys * (int)sizeof(uint32_t));
         if (e != cudaSuccess) return e;
         const unsigned grid = walk_grid(select_topm_smem<NT>, NT, key_bytes, units, 1);
         e = launch_pdl(select_topm_smem<NT>, dim3(grid), dim3(NT), key_bytes, s, scores, lens, lens_out, keep, w,

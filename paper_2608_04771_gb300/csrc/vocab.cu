@@ -508,8 +508,7 @@ cudaError_t launch_penalty_sample(float *logits, int B, int V, const int32_t *id
     const int rpc = (nrec + C - 1) / C;
     if ((V & 3) == 0 && ((uintptr_t)logits & 15u) == 0 && rpc <= kSampleClusterRecs) {
         const size_t smem = (size_t)rpc * kSampleRec * sizeof(float);
-        cudaError_t e = cudaFuncSetAttribute(sample_cluster<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kSampleClusterRecs * kSampleRec * (int)sizeof(float));
+        cudaError_t e = allow_smem((const void *)sample_cluster<256>, kSampleClusterRecs * kSampleRec * (int)sizeof(float));
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(C, B);

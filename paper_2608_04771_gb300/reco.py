@@ -93,7 +93,7 @@ def _ok(status: int):
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
@@ -102,9 +102,9 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 def _stream(stream):
     if stream is None:
         if _raw_stream is not None:  # the current stream's handle without building a Stream object
-            return ctypes.c_void_p(_raw_stream(torch.cuda.current_device()))
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
 
 
 def _dtype_code(dt):
