@@ -104,6 +104,12 @@ __device__ __forceinline__ void bulk_load_hint(uint32_t dst, const void *src, ui
         : "memory");
 }
 
+// Bulk prefetch of `bytes` (a multiple of 16, from a 16-byte boundary) into L2.
+__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(src)), "r"(bytes) : "memory");
+}
+
 // An L2 policy under which every access is evicted first (data read once).
 __device__ __forceinline__ uint64_t l2_evict_first_policy()
 {
