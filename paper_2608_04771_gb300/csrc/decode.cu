@@ -32,6 +32,7 @@
 #include <cuda.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -75,7 +76,7 @@ struct DecodeArgs {
     int units, Hq, Hkv, G, L_cap, append, out_bf16;
     float c2;  // scale * log2(e)
     unsigned *err;
-    int gv;           // query heads per virtual unit (half of G where a unit runs as two)
+    int hs_min, hs_max;  // virtual units per unit, each of G / hs query heads
     float *ring;      // or nullptr: lse rows ring[*slot] and ring[*slot + slots], each [nq]
     long long *slot;  // device ring row, advanced by one (mod slots) per launch
     int slots;
@@ -270,6 +271,7 @@ constexpr long long kSpinLimit = 1LL << 24;  // bounded mbarrier waits (about a 
 constexpr float kLazyLog2 = 8.f;             // output rescale threshold (log2 units)
 constexpr int kMinBlocksPerWarp = 4;         // fewer working warps rather than shorter ranges
 constexpr int kMaxWholeBlocks = 16;          // units of at most this many blocks are never cut
+constexpr int kOnePassBlocks = 16;           // blocks per warp from which all heads of a unit run in one pass
 constexpr int kDeepBlocksPerWarp = 64;       // from this many blocks per warp, half the warps with deep rings
 
 constexpr int kStageBytes128 = 8192;         // a block of K and V rows at d = 128 (half of it at d = 64)
@@ -303,14 +305,21 @@ __device__ __forceinline__ uint32_t swz(int rr, int ch) { return rr * 128 + ((ch
 // bf16: QK^T and PV run on mma.sync m16n8k16 with NT * 8 query heads per unit.  The QK tile has
 // 16 query rows: heads 0-7 fill its first eight, heads 8-15 (NT = 2) the others, which cost the
 // product nothing more; PV takes one 8-head column tile per NT.
-template <int D_, int NT_> struct Bf16Block {
-    static constexpr int D = D_, HS = 1, NT = NT_, KB = 16, GM = 8 * NT;
+template <class T> struct Tag {
+    using type = T;
+};
+
+template <int D_, int NT_, int HALVES_ = 1> struct Bf16Block {
+    static constexpr int D = D_, NT = NT_, KB = 16, GM = 8 * NT;
+    // units run as two halves of their heads (HALVES = 2), or may (NT = 2): then by consumer Half
+    static constexpr bool SPLIT = NT == 2 || HALVES_ == 2, ALWAYS = HALVES_ == 2;
+    using Half = Bf16Block<D_, 1, HALVES_>;
     static constexpr int ROW = 2 * D, HALVES = D / 64, TILE = 16 * 128, MT = D / 16;
     static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = 0;
     static constexpr bool TENSOR_MAPS = true, PREFETCH_Q = NT == 1;
     // half the warps with deeper rings for long work: up to eight heads a block leaves a warp
-    // waiting for data; with sixteen its arithmetic wants all the warps (160 against 155 us)
-    static constexpr bool DEEP = NT == 1;
+    // waiting for data; with more its arithmetic wants all the warps (160 against 155 us)
+    static constexpr bool DEEP = true;
 
     uint32_t qa[D / 16][2 * NT], qn[PREFETCH_Q ? D / 16 : 1][2 * NT];
     float o[NT][MT][4], m[NT], l[NT];
@@ -318,6 +327,7 @@ template <int D_, int NT_> struct Bf16Block {
     int nh_src = 0;
     const int g, c;
 
+    static_assert(NT_ == 1 || HALVES_ == 1, "sixteen heads need no halves");
     __device__ __forceinline__ Bf16Block(int lane, float *) : g(lane >> 2), c(lane & 3) {}
 
     __device__ static __forceinline__ uint32_t chunk(int row, int ch) { return (ch >> 3) * TILE + swz(row, ch & 7); }
@@ -531,14 +541,16 @@ template <int D_, int NT_> struct Bf16Block {
     }
 };
 
-// float32: plain FMAs in float32 throughout, GT >= G (or half of G, HS = 2) query heads.  In QK^T
+// float32: plain FMAs in float32 throughout, GT >= G (or half of G) query heads.  In QK^T
 // lane (kq = lane / 8, part = lane % 8) holds D / 8 elements of every head's query (32-element
 // groups, four at part * 4) and multiplies them with keys kq and kq + 4 of the block; the eight
 // parts are then added by halving exchanges that leave each (key, head) sum in one lane.  In PV a
 // lane owns D / 32 columns of every head's output and takes the probabilities from shared memory.
-template <int D_, int GT_, int HS_> struct F32Block {
-    static constexpr int D = D_, HS = HS_, KB = 8, GM = GT_, GT = GT_, E = D / 32, QE = D / 8;
+template <int D_, int GT_> struct F32Block {
+    static constexpr int D = D_, KB = 8, GM = GT_, GT = GT_, E = D / 32, QE = D / 8;
     static constexpr int ROW = 4 * D;
+    static constexpr bool SPLIT = GT == 8, ALWAYS = false;  // units of more than 8 heads run as two halves
+    using Half = F32Block;
     static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = KB * GT;
     static constexpr bool TENSOR_MAPS = false;
     static constexpr bool DEEP = false;  // bound by its arithmetic: all the warps (93 against 70 us)
@@ -767,7 +779,7 @@ template <class Block>
 __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     decode_stream(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, DecodeArgs a)
 {
-    constexpr int D = Block::D, HS = Block::HS, KB = Block::KB, GM = Block::GM;
+    constexpr int D = Block::D, KB = Block::KB;
     using LY = RingLayout<D>;
     constexpr int NW = kDecodeWarps, S = kDecodeStages;
     constexpr int STAGE = LY::STAGE;
@@ -781,7 +793,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     const uint32_t ring0 = (raw0 + 1023u) & ~1023u;
     int *sm_pre = reinterpret_cast<int *>(smem_raw + (ring0 - raw0) + LY::RING);  // [units + 1]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int units = a.units;
+    const int P = a.units;  // cache units
     if (Block::TENSOR_MAPS && tid == 0) {  // fetch both descriptors (kernel parameters) while the previous kernel drains
         prefetch_tensormap(&tmK);
         prefetch_tensormap(&tmV);
@@ -803,33 +815,22 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // (<= kMaxWholeBlocks blocks) are never cut: a range start inside one moves to the
     // unit's nearer end, since there a merge costs more than the imbalance it removes.
     int *pb = sm_pre;  // [units + 1] prefix of blocks
-    const int seg = (units + blockDim.x - 1) / blockDim.x;
-    const int u_lo = min(units, tid * seg), u_hi = min(units, u_lo + seg);
-    // Units here are virtual: unit u covers query heads [(u / P) * gv, ...) of the cache
-    // unit u % P (P cache units).  With two halves (G > 8) all first halves come first in
-    // the plan, then all second halves in the same order, so warps w and w + W/2 stream
-    // the same rows at about the same time and the second read mostly hits L2.
-    const int GS = a.gv, P = units / HS;
-    auto cache_unit = [&](int u) { return HS == 1 ? u : u % P; };
-    auto head_part = [&](int u) { return HS == 1 ? 0 : u / P; };
-    auto eff_len = [&](int u) {
-        const int L = a.lens[cache_unit(u)];
-        return unit_ok(L, a.L_cap, a.append) ? L + a.append : -1;
-    };
+    const int seg = (P + blockDim.x - 1) / blockDim.x;
+    const int u_lo = min(P, tid * seg), u_hi = min(P, u_lo + seg);
     // stage the lengths in the (still idle) ring memory with one coalesced sweep; the
     // plan below reads them from there (the ring is first written by TMA after the plan)
     int *len_sm = reinterpret_cast<int *>(smem_raw + (ring0 - raw0));
-    for (int u0 = 0; u0 < units; u0 += 8 * (int)blockDim.x) {
+    for (int u0 = 0; u0 < P; u0 += 8 * (int)blockDim.x) {
         int Lr[8];  // all loads of the batch in flight before any store or error report
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int u = u0 + k * (int)blockDim.x + tid;
-            Lr[k] = u < units ? __ldcg(a.lens + cache_unit(u)) : 0;
+            Lr[k] = u < P ? __ldcg(a.lens + u) : 0;
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int u = u0 + k * (int)blockDim.x + tid;
-            if (u < units) {
+            if (u < P) {
                 const bool ok = unit_ok(Lr[k], a.L_cap, a.append);
                 if (!ok && blockIdx.x == 0)
                     raise_error(a.err, (a.append && Lr[k] == a.L_cap) ? ERR_ROOM : ERR_LEN);
@@ -842,7 +843,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // a unit's first rows: each CTA sends its share of the units' first two blocks to L2 now (1792
     // units of 40 to 200 rows 32.7 -> 30.5 us, of 200 to 600 rows 78.2 -> 77.2 us; four blocks 31.8;
     // with fewer units than half the warps nothing changes).
-    if (2 * units >= (int)gridDim.x * NW)
+    if (2 * P >= (int)gridDim.x * NW)
         for (int u = blockIdx.x + tid * gridDim.x; u < P; u += blockDim.x * gridDim.x) {
             const int rows = min(len_sm[u] - a.append, 2 * KB);  // rows in the cache
             if (rows <= 0) continue;
@@ -878,11 +879,41 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
             pb[u] = rb;
             rb += (len_sm[u] + KB - 1) / KB;
         }
-        if (tid == blockDim.x - 1) pb[units] = rb;
+        if (tid == blockDim.x - 1) pb[P] = rb;
     }
     __syncthreads();
-    const int NB = pb[units];
     const int total_warps = gridDim.x * NW;
+    int max_nb = 0, n_ne = 0;  // most blocks of one unit; units with keys
+#pragma unroll
+    for (int w2 = 0; w2 < NW; ++w2) {
+        max_nb = max(max_nb, sm_red[w2]);
+        n_ne += sm_red[NW + w2];
+    }
+    // Units of more than 8 query heads may run as two virtual units of half the heads over the same
+    // rows (float32 always does).  One pass over a block for all heads costs less than two when the
+    // warps are busy with blocks; with few blocks per warp, twice as many units keep more warps busy
+    // and their merges are half as large.  Measured (one pass against halves, us): 448 units of 2000
+    // to 4100 rows 142 : 217, 1456 of 187 to 750 80 : 116, 648 of 328 44 : 41, 450 of 272 to 818
+    // 54 : 47, 198 of 525 46 : 37, 8 of 12000 to 24000 331 : 84.
+    const int hs = !Block::SPLIT ? 1 : (Block::ALWAYS ? 2 : (pb[P] >= kOnePassBlocks * total_warps ? a.hs_min : a.hs_max));
+    // Virtual unit u covers half u / P (of gv heads) of the cache unit u % P: all first halves come
+    // first in the plan, then all second halves in the same order, so warps w and w + W/2 stream
+    // the same rows at about the same time and the second read mostly hits L2.
+    const int units = Block::SPLIT ? hs * P : P, GS = Block::SPLIT ? (a.G + hs - 1) / hs : a.G;
+    auto cache_unit = [&](int u) { return Block::SPLIT && u >= P ? u - P : u; };
+    auto head_part = [&](int u) { return Block::SPLIT && u >= P ? 1 : 0; };
+    auto eff_len = [&](int u) {
+        const int L = a.lens[cache_unit(u)];
+        return unit_ok(L, a.L_cap, a.append) ? L + a.append : -1;
+    };
+    const int NB = (Block::SPLIT ? hs : 1) * pb[P];
+    n_ne *= Block::SPLIT ? hs : 1;
+    if (Block::SPLIT && hs == 2) {
+        __syncthreads();  // pb[P] has been read
+        for (int u = u_lo; u < u_hi; ++u) pb[P + u] = NB / 2 + pb[u];
+        if (tid == blockDim.x - 1) pb[units] = NB;
+        __syncthreads();
+    }
     // Long work (at least kDeepBlocksPerWarp blocks per warp) runs on half the warps, each
     // with a ring twice as deep: more bytes in flight per warp keep HBM busier once every
     // warp has many blocks; short work keeps all warps for latency.  The CTA's ring is the
@@ -890,14 +921,8 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // Fewer than half as many units as warps (with at least 8 blocks per warp) also
     // takes the deep partition: there the 8-warp split would cut every unit into many
     // pieces, whose merges cost more than the shallower rings save.
-    const bool deep = Block::DEEP && (NB >= kDeepBlocksPerWarp * total_warps ||
+    const bool deep = Block::DEEP && GS <= 8 && (NB >= kDeepBlocksPerWarp * total_warps ||
                                       (NB >= 8 * total_warps && total_warps > 2 * units));
-    int max_nb = 0, n_ne = 0;  // most blocks of one unit; units with keys
-#pragma unroll
-    for (int w2 = 0; w2 < NW; ++w2) {
-        max_nb = max(max_nb, sm_red[w2]);
-        n_ne += sm_red[NW + w2];
-    }
     // Only short units (none is ever cut): the contiguous deal below would leave some warps
     // two whole units where others have one.  Instead the units are sorted by blocks, most
     // first (ties by index, so every CTA builds the same order), and dealt in snake order:
@@ -909,9 +934,9 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     int *order = sm_pre;
     if (snake) {
         constexpr int NBK = kMaxWholeBlocks + 1;  // buckets: 16 - blocks, so most blocks first
-        int *cnt = len_sm + ((units + 31) & ~31);  // [NBK][blockDim.x], also in the idle ring
+        int *cnt = len_sm + ((P + 31) & ~31);  // [NBK][blockDim.x], also in the idle ring
         for (int k = 0; k < NBK; ++k) cnt[k * blockDim.x + tid] = 0;
-        for (int u = u_lo; u < u_hi; ++u) ++cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid];
+        for (int u = u_lo; u < u_hi; ++u) cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid] += Block::SPLIT ? hs : 1;
         __syncthreads();
         // exclusive scan of cnt in memory order (bucket-major, then thread): thread t takes
         // entries [NBK t, NBK (t + 1))
@@ -935,15 +960,27 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         }
         __syncthreads();
         // each thread places its own units, in index order, from its own column of cnt
-        for (int u = u_lo; u < u_hi; ++u) order[cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid]++] = u;
+        for (int u = u_lo; u < u_hi; ++u) {
+            int &at = cnt[(kMaxWholeBlocks - ((len_sm[u] + KB - 1) / KB)) * blockDim.x + tid];
+            order[at++] = u;
+            if (Block::SPLIT && hs == 2) order[at++] = P + u;
+        }
         __syncthreads();
     }
     bool aborted = false;
-    {
+    // the warp's items, by block consumer C
+    auto run = [&](auto tag) {
+    using C = typename decltype(tag)::type;
+    constexpr int GM = C::GM;
     const int NWm = deep ? NW / 2 : NW, Sm = deep ? 2 * S : S;  // NWm * Sm == NW * S either way
     const uint32_t my_ring = ring0 + (uint32_t)wid * Sm * STAGE;
-    // working warps: every one gets at least kMinBlocksPerWarp blocks (or all warps work)
-    const int W = max(1, min(NWm * (int)gridDim.x, NB / kMinBlocksPerWarp));
+    // Working warps: every one gets at least kMinBlocksPerWarp blocks (or all warps work), and few
+    // units are cut into few pieces: one warp merges a unit's pieces one after another, each at about
+    // the cost of a block, so pieces per unit do not exceed blocks per warp, W^2 <= NB * units
+    // (2 units of 32000 rows, 7 heads: 341 us on all warps, 74 so, 100 with sqrt(5) times as many;
+    // from some 40 long units on every warp works).
+    int W = max(1, min(NWm * (int)gridDim.x, NB / kMinBlocksPerWarp));
+    while (W > 1 && (long long)W * W > (long long)NB * n_ne) W -= max(1, W >> 4);
     const bool out_bf16 = a.out_bf16 != 0;
     auto wstart = [&](int w) { return (int)((long long)w * NB / W); };  // ideal first block of warp w
     auto owner = [&](int b) { return (int)(((long long)(b + 1) * W - 1) / NB); };  // ideal owner of block b
@@ -1070,7 +1107,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         return it;
     };
 
-    Block blk(lane, Block::SCRATCH > 0 ? sm_block + wid * Block::SCRATCH : nullptr);
+    C blk(lane, C::SCRATCH > 0 ? sm_block + wid * C::SCRATCH : nullptr);
     auto load_q = [&](const Item &it) {
         const long qrow = (long)(it.pu / a.Hkv) * a.Hq + (long)(it.pu % a.Hkv) * a.G + it.hp * GS;
         blk.load_q(a.q, qrow, min(GS, a.G - it.hp * GS));
@@ -1315,6 +1352,13 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
             pblk = 0;
         }
     }
+    };
+    if constexpr (std::is_same_v<Block, typename Block::Half>) {  // one consumer
+        run(Tag<Block>{});
+    } else if (GS > 8) {
+        run(Tag<Block>{});
+    } else {
+        run(Tag<typename Block::Half>{});
     }
 
     // Every warp, stopped early or not, counts itself done with one 64-bit add on the
@@ -1340,7 +1384,7 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
             // 16 independent loads per lane in flight before any store, of 4 lengths each
             // when lens is 16-byte aligned: one L2 round trip for up to 2048 units
             constexpr int BATCH = 16;
-            const int cu = units / HS;  // cache units
+            const int cu = P;  // cache units
             const int n4 = (reinterpret_cast<uintptr_t>(a.lens) & 15u) == 0 ? cu / 4 : 0;
             int4 *l4 = reinterpret_cast<int4 *>(a.lens);
             for (int i0 = 0; i0 < n4; i0 += 32 * BATCH) {
@@ -1412,16 +1456,22 @@ static bool encode_cache_map(CUtensorMap *map, const void *base, unsigned long l
 
 typedef void (*DecodeKernel)(CUtensorMap, CUtensorMap, DecodeArgs);
 
-// float32 kernel for up to gt (2, 4, 6 or 8) query heads per virtual unit, hs of them per unit.
-template <int D> static DecodeKernel f32_kernel(int gt, int hs)
+// float32 kernel for up to gt (2, 4, 6 or 8) query heads per virtual unit.
+template <int D> static DecodeKernel f32_kernel(int gt)
 {
-    if (hs == 2) return decode_stream<F32Block<D, 8, 2>>;
     switch (gt) {
-    case 2: return decode_stream<F32Block<D, 2, 1>>;
-    case 4: return decode_stream<F32Block<D, 4, 1>>;
-    case 6: return decode_stream<F32Block<D, 6, 1>>;
-    default: return decode_stream<F32Block<D, 8, 1>>;
+    case 2: return decode_stream<F32Block<D, 2>>;
+    case 4: return decode_stream<F32Block<D, 4>>;
+    case 6: return decode_stream<F32Block<D, 6>>;
+    default: return decode_stream<F32Block<D, 8>>;
     }
+}
+
+// bf16 kernel: up to 8 query heads per unit, or up to 16, of which `halves` makes two units.
+template <int D> static DecodeKernel bf16_kernel(bool wide, bool halves)
+{
+    if (!wide) return decode_stream<Bf16Block<D, 1>>;
+    return halves ? decode_stream<Bf16Block<D, 1, 2>> : decode_stream<Bf16Block<D, 2>>;
 }
 
 cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, const void *v_new,
@@ -1458,16 +1508,20 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
     a.nq_rows = a.nq;
     a.advance = 1;
     const bool f32 = kv.dtype == RECO_F32;
-    // query heads per virtual unit: float32 units of more than 8 heads run as two of half as many
+    // virtual units per unit: float32 units of more than 8 heads run as two of half as many; bf16
+    // ones may (the kernel decides from the lengths), as long as one plan holds all units twice
     const int hs = f32 && a.G > 8 ? 2 : 1;
-    a.gv = (a.G + hs - 1) / hs;
+    a.hs_min = hs;
     DecodeKernel fn;
     if (f32) {
-        const int gt = std::min(8, (a.gv + 1) / 2 * 2);
-        fn = kv.d == 64 ? f32_kernel<64>(gt, hs) : f32_kernel<128>(gt, hs);
+        const int gt = a.G > 6 ? 8 : (a.G + 1) / 2 * 2;  // (halves of more than 8 heads: by the widest)
+        fn = kv.d == 64 ? f32_kernel<64>(gt) : f32_kernel<128>(gt);
     } else {
-        fn = kv.d == 64 ? (a.G > 8 ? decode_stream<Bf16Block<64, 2>> : decode_stream<Bf16Block<64, 1>>)
-                        : (a.G > 8 ? decode_stream<Bf16Block<128, 2>> : decode_stream<Bf16Block<128, 1>>);
+        // With more than 8 heads: a cache that cannot hold 24 blocks a warp runs as halves in any case
+        // (the kernel of one consumer is up to 10% faster there than the one that may choose).
+        const bool halves = a.G > 8 && 2LL * std::min<long long>(a.units, kMaxTmaUnits) <= kMaxTmaUnits &&
+                            (long long)a.units * ((kv.L_cap + 15) / 16) < 24LL * kDecodeWarps * device_sm_count();
+        fn = kv.d == 64 ? bf16_kernel<64>(a.G > 8, halves) : bf16_kernel<128>(a.G > 8, halves);
     }
     // More units than one plan holds in shared memory run as consecutive launches over
     // contiguous unit ranges (every unit is independent): each part gets its own K/V, q,
@@ -1488,8 +1542,9 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
                 if (u0 == 0) break;  // the SIMT path below takes the whole call
                 return cudaErrorInvalidValue;
             }
-            DecodeArgs at = a;  // virtual units of this part
-            at.units = (int)(cu * hs);
+            DecodeArgs at = a;  // this part
+            at.units = (int)cu;
+            at.hs_max = a.G > 8 && 2 * cu <= (f32 ? kMaxF32Units : kMaxTmaUnits) ? 2 : hs;
             at.K = const_cast<char *>(kb);
             at.V = const_cast<char *>(vb);
             at.q = static_cast<const char *>(q) + (size_t)q0 * row_b;
@@ -1503,7 +1558,8 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
             at.nq_rows = cu * a.G;
             at.advance = u0 + cu >= a.units ? 1 : 0;
             // the counters are zero on entry (zero-filled workspace) and every launch leaves them so
-            const size_t smem = kv.d == 64 ? ring_smem_bytes<64>(at.units) : ring_smem_bytes<128>(at.units);
+            const int plan = at.units * at.hs_max;
+            const size_t smem = kv.d == 64 ? ring_smem_bytes<64>(plan) : ring_smem_bytes<128>(plan);
             cudaError_t e = allow_smem((const void *)fn, (int)smem);
             if (e != cudaSuccess) return e;
             // two partial slots per warp of the grid
@@ -1514,7 +1570,6 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
         }
     }
     // bf16 caches that no tensor map covers
-    a.gv = a.G;
     const unsigned grid = (unsigned)a.units;
     if (kv.d == 64) decode_simt<__nv_bfloat16, 64><<<grid, 128, 0, s>>>(a);
     else decode_simt<__nv_bfloat16, 128><<<grid, 128, 0, s>>>(a);
