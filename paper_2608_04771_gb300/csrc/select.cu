@@ -7,7 +7,7 @@
 // largest key T and how many keys equal to T are still needed; one ordered pass then emits every
 // candidate with key > T plus the first `need` with key == T in index order.  The result is
 // sorted and ties go to the lower index, with no sort.
-//   select_topm_warp  up to 1024: one warp per unit, keys in registers
+//   select_topm_warp  up to 256, and up to 1024 where there are many units: one warp per unit, keys in registers
 //   select_topm_smem  up to kSelectSmemKeys: CTAs walk the units, keys in shared memory
 //   select_topm       longer: CTAs walk the units, keys read from global memory
 // A unit whose sequence keeps its whole cache is an identity, skipped by the compaction.
@@ -203,13 +203,19 @@ __global__ void __launch_bounds__(NT) select_topm(const float *__restrict__ scor
     }
 }
 
+// The search ends as soon as a prefix splits off exactly the keys still needed: every key at or above
+// it is taken, so equal ones need no count.  Neighbouring scores among n differ some log2(n) + 2 bits
+// below their range, which leaves half of the 25 or so bits unread: 304 units of 264 rows 5.2 -> 3.9 us,
+// 1030 rows by warps 16.3 -> 9.5, 1216 units of 16400 rows 70 -> 65.
+constexpr int kWholeBin = 0x7fffffff;
+
 // The same selection with the unit's keys staged in shared memory once (all loads in flight), the
 // radix passes run from there, and the ordered emit done by warp-contiguous segments: one counting
 // sweep, one scan of the warps' counts, one writing sweep.  The passes start below the bits that
 // all keys share (their smallest and largest key): scores of one unit lie within a few powers of
 // two, so a first digit of the top eight bits put nearly all keys into two or three bins, whose
-// atomics serialise.  512 threads, so that three units of 16384 keys share an SM and one counts
-// while another waits at a barrier.  512 units of 15000 to 16384 candidates: 54 -> 45 us.
+// atomics serialise.  Where there are more units than SMs, smaller CTAs share an SM and one counts
+// while another waits at a barrier (512 units of 15000 to 16384 candidates: 54 -> 45 us).
 template <int NT>
 __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__ scores, const int32_t *lens,
                                                        int32_t *lens_out, const int32_t *__restrict__ keep, int w, int B, int Hkv,
@@ -227,6 +233,7 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
     __shared__ int2 s_lm[kWalkAhead];
     wait_prior_grid();  // scores, lens and keep may come from the previous kernels
     walk_headers(s_lm, lens, keep, units, B, Hkv);
+    for (int i = threadIdx.x; i < 256; i += NT) hist[i] = 0;
     __syncthreads();
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int it = 0;
@@ -273,8 +280,6 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
             int remaining = kc;
             while (bits > 0) {
                 const int shift = max(0, bits - 8);
-                for (int i = tid; i < 256; i += NT) hist[i] = 0;
-                __syncthreads();
                 for (int j = tid; j < nc; j += NT) {
                     const uint32_t key = keys[j];
                     // plain shared-memory atomics: grouping a warp's equal bins first
@@ -282,11 +287,12 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
                     if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
                 }
                 __syncthreads();
-                if (wid == 0) {  // find the bin holding the remaining-th largest key
+                if (wid == 0) {  // find the bin holding the remaining-th largest key; clear for the next pass
                     int c8[8], sum = 0;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         c8[i] = hist[255 - 8 * lane - i];
+                        hist[255 - 8 * lane - i] = 0;
                         sum += c8[i];
                     }
                     int incl = sum;
@@ -301,7 +307,7 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
                         for (int i = 0; i < 8; ++i) {
                             if (cum + c8[i] >= remaining) {
                                 s_prefix = (uint32_t)(255 - 8 * lane - i) << shift;
-                                s_remaining = remaining - cum;
+                                s_remaining = c8[i] == remaining - cum ? kWholeBin : remaining - cum;
                                 break;
                             }
                             cum += c8[i];
@@ -312,6 +318,7 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
                 // a first digit of fewer than eight bits meets bins of the shared bits above them
                 prefix |= s_prefix;
                 remaining = s_remaining;
+                if (remaining == kWholeBin) break;
                 mask |= 255u << shift;
                 bits = shift;
             }
@@ -382,8 +389,8 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
 // The same selection for short units (L_cap - w <= 32 * K): one warp per unit, its keys in
 // registers (lane l holds candidates l, l + 32, ...), the threshold found bit by bit from the top
 // one in which keys differ: a count of the keys at or above each trial value, no shared memory and
-// no barrier.  A CTA of 512 threads spends such a unit's time at its barriers (step boundary of
-// the trace, 1792 units of 90 to 240 rows, one eighth of them compressed: 14 -> 9 us).
+// no barrier.  A CTA spends such a unit's time at its barriers (step boundary of
+// the trace, 1792 units of 90 to 240 rows, one eighth of them compressed: 14 -> 9 us before the early end above).
 constexpr int kWarpThreads = 256;
 
 template <int K>
@@ -436,12 +443,19 @@ __global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__
             int n[4] = {0, 0, 0, 0};
 #pragma unroll
             for (int i = 0; i < K; ++i) n[i & 3] += key[i] >= trial;
-            if (__reduce_add_sync(0xffffffffu, (n[0] + n[1]) + (n[2] + n[3])) >= kc) T = trial;
+            const int at = __reduce_add_sync(0xffffffffu, (n[0] + n[1]) + (n[2] + n[3]));
+            if (at >= kc) T = trial;
+            if (at == kc) {
+                need = kWholeBin;
+                break;
+            }
         }
-        int n = 0;
+        if (need == 0) {
+            int n = 0;
 #pragma unroll
-        for (int i = 0; i < K; ++i) n += key[i] > T;
-        need = kc - __reduce_add_sync(0xffffffffu, n);
+            for (int i = 0; i < K; ++i) n += key[i] > T;
+            need = kc - __reduce_add_sync(0xffffffffu, n);
+        }
     }
     const unsigned below = (1u << lane) - 1u;
     int e_run = 0, pos = 0;
@@ -586,14 +600,31 @@ static unsigned walk_grid(F fn, int threads, size_t smem, long units, int per_un
     return (unsigned)std::min(units, ctas);
 }
 
+template <int NT>
+static cudaError_t launch_select_smem(const reco_kv &kv, size_t key_bytes, long units, const float *scores,
+                                      const int32_t *lens, int32_t *lens_out, const int32_t *keep, int w, int32_t *idx,
+                                      int32_t *count, unsigned *err, cudaStream_t s)
+{
+    const cudaError_t e =
+        allow_smem((const void *)select_topm_smem<NT>, (int)kSelectSmemKeys * (int)sizeof(uint32_t));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(select_topm_smem<NT>, dim3(walk_grid(select_topm_smem<NT>, NT, key_bytes, units, 1)), dim3(NT),
+                      key_bytes, s, scores, lens, lens_out, keep, w, kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
+}
+
 static cudaError_t launch_select(const reco_kv &kv, const float *scores, const int32_t *lens, int32_t *lens_out,
                                  const int32_t *keep, int w, int32_t *idx, int32_t *count, unsigned *err,
                                  cudaStream_t s)
 {
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
     const int most = kv.L_cap - w;  // candidates of a unit
+    const int sms = device_sm_count();
     cudaError_t e;
-    if (most <= 32 * 32) {  // short units: a warp each
+    // A warp per unit costs 3.5 to 4 us up to 256 candidates, 6 up to 512 and 9.5 up to 1024, whatever the
+    // number of units (its lanes hold 8, 16 or 32 keys one after another), against 4.2 at best for a CTA
+    // per unit, which grows with the units: 520 rows, 304 units 5.9 by warps and 5.1 by CTAs, 608 units
+    // 6.0 and 6.0, 1216 units 6.1 and 9.5; 1030 rows, 608 units 9.5 and 7.5, 1216 units 9.5 and 11.6.
+    if (most <= 32 * 8 || (most <= 32 * 32 && units > (most <= 32 * 16 ? 4L : 6L) * sms)) {
         auto fn = most <= 32 * 8 ? select_topm_warp<8> : (most <= 32 * 16 ? select_topm_warp<16> : select_topm_warp<32>);
         constexpr int per = kWarpThreads / 32;
         e = launch_pdl(fn, dim3((unsigned)((units + per - 1) / per)), dim3(kWarpThreads), 0, s, scores, lens, lens_out,
@@ -604,12 +635,16 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
     // keys of a unit staged in shared memory when L_cap - w of them fit
     const size_t key_bytes = (size_t)most * sizeof(uint32_t);
     if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
-        constexpr int NT = 512;
-        e = allow_smem((const void *)select_topm_smem<NT>, (int)kSelectSmemKeys * (int)sizeof(uint32_t));
-        if (e != cudaSuccess) return e;
-        const unsigned grid = walk_grid(select_topm_smem<NT>, NT, key_bytes, units, 1);
-        e = launch_pdl(select_topm_smem<NT>, dim3(grid), dim3(NT), key_bytes, s, scores, lens, lens_out, keep, w,
-                       kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
+        // Threads per unit: as many as let all units be resident at once, within what a unit can use.
+        // us with 256 / 512 / 1024 threads: 152 units of 4100 rows 10.9 / 8.9 / 7.7, of 1030 rows 6.9 / 5.8 / 6.3;
+        // 304 units of 4100 rows 11.3 / 10.1 / 10.2; 1216 units of 4100 rows 22.6 / 24.4 / 33.1, of 16400 rows
+        // 79 / 65 / 72 (there the keys, not the threads, bound the units an SM holds).
+        if (units <= sms && most > 1024)
+            e = launch_select_smem<1024>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
+        else if (units <= 2L * sms || most > 6 * 1024)
+            e = launch_select_smem<512>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
+        else
+            e = launch_select_smem<256>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
         if (e != cudaSuccess) return e;
     } else {
         const unsigned grid = walk_grid(select_topm<1024>, 1024, 0, units, 1);

@@ -1,5 +1,6 @@
-"""The top-m selection's kernels by unit length (a warp per unit up to 256, 512 and 1024 candidates,
-shared memory above), bit for bit against the oracle on scores that stress the radix digits: ties,
+"""The top-m selection's kernels by unit length and number of units (a warp per unit up to 256
+candidates, up to 512 with more than 4 units per SM and up to 1024 with more than 6; else CTAs of 256, 512 and 1024
+threads), bit for bit against the oracle on scores that stress the radix digits: ties,
 equal scores, neighbours one ulp apart, all magnitudes and signs, infinities."""
 import numpy as np
 import pytest
@@ -34,12 +35,18 @@ def _patterns(rng, n):
     ]
 
 
-@pytest.mark.parametrize("most", [1, 5, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000, 9001])
-def test_selection_by_length(most):
-    rng = np.random.default_rng(most)
+SMS = 152
+
+
+@pytest.mark.parametrize("B,most", [(16, m) for m in (1, 5, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000, 9001)]
+                         + [(B, m) for B in (SMS // 2, SMS // 2 + 1, SMS, SMS + 1) for m in (257, 1024, 1025)]
+                         + [(SMS + 1, 6144), (SMS + 1, 6145)]
+                         + [(B, m) for B in (2 * SMS, 2 * SMS + 1, 3 * SMS, 3 * SMS + 1) for m in (257, 512, 513, 1024)])
+def test_selection_by_length(B, most):
+    rng = np.random.default_rng(most + 10007 * (B - 16))
     w = 5
     L_cap = most + w
-    B, H = 16, 2
+    H = 2
     lens = np.zeros((1, B, H), np.int32)
     keep = np.zeros(B, np.int32)
     scores = np.zeros((1, B, H, L_cap), np.float32)
