@@ -635,13 +635,16 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
     // keys of a unit staged in shared memory when L_cap - w of them fit
     const size_t key_bytes = (size_t)most * sizeof(uint32_t);
     if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
-        // Threads per unit: as many as let all units be resident at once, within what a unit can use.
-        // us with 256 / 512 / 1024 threads: 152 units of 4100 rows 10.9 / 8.9 / 7.7, of 1030 rows 6.9 / 5.8 / 6.3;
-        // 304 units of 4100 rows 11.3 / 10.1 / 10.2; 1216 units of 4100 rows 22.6 / 24.4 / 33.1, of 16400 rows
-        // 79 / 65 / 72 (there the keys, not the threads, bound the units an SM holds).
-        if (units <= sms && most > 1024)
+        // Threads per unit, by how many units an SM can hold (as their keys allow) and has to: larger CTAs
+        // are faster for one unit, smaller ones let one unit count while another waits at a barrier.  us with
+        // 256 / 512 / 1024 threads: 1 unit per SM of 4100 rows 10.9 / 8.9 / 7.7, of 1030 rows 6.9 / 5.8 / 6.3;
+        // 2 of 4100 rows 11.3 / 10.1 / 10.2; 3 of 16400 rows (1216 units) 79 / 65 / 72; 4 of 6200 rows
+        // 16.6 / 16.0 / 21.5; 8 of 4100 rows 22.6 / 24.4 / 33.1; 1216 units of 32800 rows, one per SM at a
+        // time, 383 / 211 / 157.
+        const long held = (long)((227 * 1024) / (key_bytes + 4096)), per_sm = std::min((units + sms - 1) / sms, held);
+        if ((per_sm <= 1 && most > 1024) || (per_sm == 2 && most > 16 * 1024))
             e = launch_select_smem<1024>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
-        else if (units <= 2L * sms || most > 6 * 1024)
+        else if (per_sm <= 4)
             e = launch_select_smem<512>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
         else
             e = launch_select_smem<256>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);

@@ -40,8 +40,8 @@ SMS = 152
 
 @pytest.mark.parametrize("B,most", [(16, m) for m in (1, 5, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000, 9001)]
                          + [(B, m) for B in (SMS // 2, SMS // 2 + 1, SMS, SMS + 1) for m in (257, 1024, 1025)]
-                         + [(SMS + 1, 6144), (SMS + 1, 6145)]
-                         + [(B, m) for B in (2 * SMS, 2 * SMS + 1, 3 * SMS, 3 * SMS + 1) for m in (257, 512, 513, 1024)])
+                         + [(B, m) for B in (2 * SMS, 2 * SMS + 1, 3 * SMS, 3 * SMS + 1) for m in (257, 512, 513, 1024)]
+                         + [(2 * SMS + 1, 1025), (SMS, 16384), (SMS, 16385), (16, 40000)])
 def test_selection_by_length(B, most):
     rng = np.random.default_rng(most + 10007 * (B - 16))
     w = 5
