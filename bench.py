@@ -588,7 +588,7 @@ def run_gpu(args, wl):
                        "rates": "compress_tokens_s = B*L / (score + select + compact); decode_tokens_s = "
                                 "B*steps / (steps * mean decode launch), attention only",
                        "kernels": kernels, "keep_counts": [int(x) for x in hp.keep_host]},
-            "roofline": {"bound": "hbm", "kernel": "decode_tma (reco_decode_attn)", "achieved": dec_achieved,
+            "roofline": {"bound": "hbm", "kernel": "decode_stream (reco_decode_attn)", "achieved": dec_achieved,
                          "peak": hbm, "unit": "GB/s", "frac": dec_achieved / hbm, "peak_kind": peak_kind,
                          "frac_of_8TBs": dec_achieved / 8000.0,
                          "traffic": traffic, "traffic_source": traffic_src,

@@ -18,9 +18,10 @@
 //   sides) so that each thread's fragments are whole 16-byte chunks, and the swizzle makes
 //   every fragment read conflict-free.  Heads 9 to 16 of a unit fill the QK tile's other
 //   eight rows: one pass over the block instead of two units of half the heads (28 x 4 x 4
-//   units of 2000 to 4100 rows, 16 heads: 226 -> 157 us).
+//   units of 2000 to 4100 rows, 16 heads: 217 -> 145 us).  Where a warp would get under 16
+//   blocks so, the halves stay units of their own.
 //   float32: blocks of 8 keys, plain FMAs (28 x 4 x 2 units of 800 to 1500 rows, 6 heads,
-//   from one CTA per unit that took its keys one by one: 516 -> 67 us).
+//   from one CTA per unit that took its keys one by one: 514 -> 60 us).
 // A unit split over several items writes partial (max, sum, output) triples; the last
 // item to finish (atomic ticket, no waiting) merges them.  The counters live in the
 // caller's workspace, zero-filled before its first use; each launch clears what it
@@ -53,7 +54,7 @@ DecodeWs decode_ws_layout(const reco_kv &kv, void *base)
     };
     DecodeWs ws;
     ws.part_slots = kDecodePartSlots;
-    // merge tickets per unit of the TMA path, which splits a unit of G > 8 heads in two
+    // merge tickets per unit; a unit of G > 8 heads may run as two
     ws.counters = (int32_t *)take((2 + units * (G > 8 ? 2 : 1)) * 4);
     ws.part_ml = (float *)take((size_t)ws.part_slots * G * 2 * 4);
     ws.part_o = (float *)take((size_t)ws.part_slots * G * kv.d * 4);

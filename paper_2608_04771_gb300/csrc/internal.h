@@ -8,11 +8,11 @@
 
 namespace reco {
 
-// Keys per scoring work item (one CTA per (unit, chunk) in both scoring passes).
+// Keys per chunk of a unit: a tensor-core scoring pass's work item, and a row partial's keys.
 constexpr int kScoreChunk = 2048;
 // Decode (m, l, O) partial slots in the workspace: two per warp of a grid of up to
-// 256 SMs x 8 warps (the workspace size may not depend on the device; a larger grid
-// takes the SIMT path).
+// 256 SMs x 8 warps (the workspace size may not depend on the device; the grid is
+// clipped to them).
 constexpr int kDecodePartSlots = 4096;
 // Sampling: logits per pass-1 segment, and the most segments a row may have.
 constexpr int kSampleSeg = 4096;

@@ -7,7 +7,7 @@
 // summed, so the scores take two passes over K:
 //   pass 1  per (unit, key chunk): per-row running max / sum in the log2 domain
 //   combine per (unit, row): merge the chunk partials -> b_r = m_r + log2 Z_r
-//   pass 2  per (unit, key chunk): column sums  sum_r 2^(c*l_rj - b_r) / G
+//   pass 2  per (unit, key tile): column sums  sum_r 2^(c*l_rj - b_r) / G
 //   pool    per (unit, key): max over the clipped window
 // This file holds the SIMT passes used for float32 caches (and any shape the tensor-
 // core passes do not cover), the combine and pool kernels, and the launcher;
