@@ -393,33 +393,11 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
 // the trace, 1792 units of 90 to 240 rows, one eighth of them compressed: 14 -> 9 us before the early end above).
 constexpr int kWarpThreads = 256;
 
+// The kept candidates of a unit, kc of its nc <= 32 * K, into idx.
 template <int K>
-__global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__restrict__ scores, const int32_t *lens,
-                                                                 int32_t *lens_out, const int32_t *__restrict__ keep,
-                                                                 int w, int B, int Hkv, int L_cap,
-                                                                 int32_t *__restrict__ idx_out,
-                                                                 int32_t *__restrict__ count, int units, unsigned *err)
+__device__ __forceinline__ void select_in_warp(const float *__restrict__ s, int nc, int kc, int32_t *__restrict__ idx,
+                                               int lane)
 {
-    wait_prior_grid();  // scores, lens and keep may come from the previous kernels
-    const int lane = threadIdx.x & 31;
-    const int u = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5);
-    if (u >= units) return;
-    const int L = lens[u], m = keep[(u / Hkv) % B];
-    if (L < w || L > L_cap || m < w || m > L) {
-        if (lane == 0) {
-            count[u] = 0;
-            raise_error(err, (L < w || L > L_cap) ? ERR_LEN : ERR_KEEP);
-        }
-        return;
-    }
-    const int nc = L - w, kc = m - w;
-    const float *s = scores + (long)u * L_cap;
-    int32_t *idx = idx_out + (long)u * L_cap;
-    if (kc == nc) {  // keep everything: identity, nothing moves (the compaction skips it)
-        for (int j = lane; j < L; j += 32) idx[j] = j;
-        if (lane == 0) count[u] = 0;
-        return;
-    }
     uint32_t key[K], lo = 0xffffffffu, hi = 0;
 #pragma unroll
     for (int i = 0; i < K; ++i) {
@@ -470,6 +448,43 @@ __global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__
         e_run += __popc(eb);
         pos += __popc(fb);
     }
+}
+
+template <int K>
+__global__ void __launch_bounds__(kWarpThreads) select_topm_warp(const float *__restrict__ scores, const int32_t *lens,
+                                                                 int32_t *lens_out, const int32_t *__restrict__ keep,
+                                                                 int w, int B, int Hkv, int L_cap,
+                                                                 int32_t *__restrict__ idx_out,
+                                                                 int32_t *__restrict__ count, int units, unsigned *err)
+{
+    wait_prior_grid();  // scores, lens and keep may come from the previous kernels
+    const int lane = threadIdx.x & 31;
+    const int u = blockIdx.x * (kWarpThreads / 32) + (threadIdx.x >> 5);
+    if (u >= units) return;
+    const int L = lens[u], m = keep[(u / Hkv) % B];
+    if (L < w || L > L_cap || m < w || m > L) {
+        if (lane == 0) {
+            count[u] = 0;
+            raise_error(err, (L < w || L > L_cap) ? ERR_LEN : ERR_KEEP);
+        }
+        return;
+    }
+    const int nc = L - w, kc = m - w;
+    const float *s = scores + (long)u * L_cap;
+    int32_t *idx = idx_out + (long)u * L_cap;
+    if (kc == nc) {  // keep everything: identity, nothing moves (the compaction skips it)
+        for (int j = lane; j < L; j += 32) idx[j] = j;
+        if (lane == 0) count[u] = 0;
+        return;
+    }
+    // a cache's units are often far shorter than its rows (the trace's boundaries, units of 70 to 240
+    // rows in a cache of up to 1024: 9.4 -> 5.8 us each)
+    if (K > 8 && nc <= 32 * 8)
+        select_in_warp<8>(s, nc, kc, idx, lane);
+    else if (K > 16 && nc <= 32 * 16)
+        select_in_warp<16>(s, nc, kc, idx, lane);
+    else
+        select_in_warp<K>(s, nc, kc, idx, lane);
     for (int t = lane; t < w; t += 32) idx[kc + t] = nc + t;
     if (lane == 0) {
         count[u] = m;
@@ -621,7 +636,7 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
     const int sms = device_sm_count();
     cudaError_t e;
     // A warp per unit costs 3.5 to 4 us up to 256 candidates, 6 up to 512 and 9.5 up to 1024, whatever the
-    // number of units (its lanes hold 8, 16 or 32 keys one after another), against 4.2 at best for a CTA
+    // number of units (its lanes hold 8, 16 or 32 keys one after another, by the unit's own length), against 4.2 at best for a CTA
     // per unit, which grows with the units: 520 rows, 304 units 5.9 by warps and 5.1 by CTAs, 608 units
     // 6.0 and 6.0, 1216 units 6.1 and 9.5; 1030 rows, 608 units 9.5 and 7.5, 1216 units 9.5 and 11.6.
     if (most <= 32 * 8 || (most <= 32 * 32 && units > (most <= 32 * 16 ? 4L : 6L) * sms)) {
@@ -642,7 +657,7 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
         // 16.6 / 16.0 / 21.5; 8 of 4100 rows 22.6 / 24.4 / 33.1; 1216 units of 32800 rows, one per SM at a
         // time, 383 / 211 / 157.
         const long held = (long)((227 * 1024) / (key_bytes + 4096)), per_sm = std::min((units + sms - 1) / sms, held);
-        if ((per_sm <= 1 && most > 1024) || (per_sm == 2 && most > 16 * 1024))
+        if ((per_sm <= 1 && most > 2048) || (per_sm == 2 && most > 16 * 1024))
             e = launch_select_smem<1024>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
         else if (per_sm <= 4)
             e = launch_select_smem<512>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
