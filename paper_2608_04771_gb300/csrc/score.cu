@@ -240,7 +240,11 @@ __global__ void score_rowb_from_lse(const int32_t *__restrict__ lens, ScoreMask 
     const long u = i / R;
     const int r = (int)(i % R);
     const int L = lens[u];
-    if (L < w || L > L_cap || mask.skip(u, L, w, L_cap)) return;
+    if (L < w || L > L_cap) {  // no other pass of this call reports it
+        if (r == 0) raise_error(err, ERR_LEN);
+        return;
+    }
+    if (mask.skip(u, L, w, L_cap)) return;
     const int g = r / w, t = r % w;
     const long qi = (u / Hkv) * Hq + (u % Hkv) * G + g;
     const float lse = row_lse[(long)t * rows_q + qi];

@@ -25,8 +25,9 @@ struct TilePlan {
 };
 
 // Runs skip .. skip + kPlanRuns of this CTA's range into pl.run; returns the range's runs.
-// Given ulist, CTA 0 also lists every unit with work (ascending) and their count.  All
-// threads of the CTA call it; it starts and ends with a CTA barrier.
+// Given ulist, CTA 0 also lists every unit with work (ascending) and their count; given err_len, it
+// reports lengths out of range, also of units that the mask leaves out.  All threads of the CTA call
+// it; it starts and ends with a CTA barrier.
 __device__ __forceinline__ int plan_runs(TilePlan &pl, const int32_t *__restrict__ lens, const ScoreMask &mask, int w,
                                          int L_cap, int units, bool candidates_only, int item_keys, int skip,
                                          int32_t *ulist, int32_t *ucount, unsigned *err_len)
@@ -34,11 +35,12 @@ __device__ __forceinline__ int plan_runs(TilePlan &pl, const int32_t *__restrict
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
     const int seg = (units + nt - 1) / nt;
     const int u_lo = min(units, tid * seg), u_hi = min(units, u_lo + seg);
+    bool bad = false;  // a length out of range: reported after the sweep, whose loads an atomic would hold back
     auto keys_of = [&](int u, int &L) {
         L = lens[u];
         const int kp = mask.keep != nullptr ? mask.keep[(u / mask.Hkv) % mask.B] : 0;  // (its load does not wait for the length)
         if (L < w || L > L_cap) {
-            if (err_len != nullptr && blockIdx.x == 0 && skip == 0) raise_error(err_len, ERR_LEN);
+            bad = true;
             return 0;
         }
         if (mask.keep != nullptr && kp >= L) return 0;
@@ -52,6 +54,7 @@ __device__ __forceinline__ int plan_runs(TilePlan &pl, const int32_t *__restrict
         my_i += (k + item_keys - 1) / item_keys;
         my_n += k > 0;
     }
+    if (bad && err_len != nullptr && blockIdx.x == 0 && skip == 0) raise_error(err_len, ERR_LEN);
     int fi = my_i, fn = my_n;  // inclusive scans within the warp
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

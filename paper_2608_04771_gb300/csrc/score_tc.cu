@@ -585,7 +585,9 @@ __global__ void __launch_bounds__(64 + 128 * kP2Groups, 1)
             }
     };
     for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
-        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, nullptr);
+        // with the normalisers given, this is the call's only pass: it reports lengths out of range
+        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount,
+                           row_lse != nullptr ? err : nullptr);
         const int n_here = min(kPlanRuns, n_runs - skip);
         if (warp == 0) {  // producer
             const int qbox_rows = NQ > 256 ? NQ / 2 : NQ;

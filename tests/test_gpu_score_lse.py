@@ -157,6 +157,28 @@ def test_non_finite_normaliser_sets_device_error():
     reco.reco_check()
 
 
+@pytest.mark.parametrize("masked", [False, True])
+@pytest.mark.parametrize("dtype,bad", [("bf16", "long"), ("bf16", "short"), ("f32", "long"), ("f32", "short")])
+def test_lse_bad_length_sets_device_error(dtype, bad, masked):
+    """A length outside [w, L_cap] is reported, also in a sequence that the mask leaves out, and its
+    unit's scores stay as they were; the other units are scored."""
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=2, L=300, decode_steps=4, dtype=dtype)
+    Kf, Vf, q_win, lens_f, _ = _window_case(wl, np.full((1, 2, wl.h_kv), 200, np.int32))
+    row_lse = torch.full((wl.w, 1, 2, wl.h_q), 5.0, dtype=torch.float32, device=DEV)
+    keep = torch.tensor([1 << 30, wl.w], dtype=torch.int32, device=DEV) if masked else None
+    good = _score_lse(wl, Kf, Vf, q_win, torch.from_numpy(lens_f).to(DEV), row_lse, keep=keep, fill=-3.0)
+    reco.reco_check()
+    lens_f[0, 0, 1] = wl.L_cap + 1 if bad == "long" else wl.w - 1
+    got = _score_lse(wl, Kf, Vf, q_win, torch.from_numpy(lens_f).to(DEV), row_lse, keep=keep, fill=-3.0)
+    with pytest.raises(reco.RecoError) as e:
+        reco.reco_check()
+    assert e.value.status == reco.RECO_EDEVICE and "length" in str(e.value)
+    assert torch.all(got[0, 0, 1] == -3.0)
+    good[0, 0, 1] = -3.0
+    assert torch.equal(got, good)
+    reco.reco_check()
+
+
 def test_lse_push_ring_and_slot():
     """Each push writes its ring row and the mirror row `slots` further on at the device slot
     and advances the slot modulo `slots` (bit-exact copies), so the last w pushes are the
