@@ -318,7 +318,9 @@ __global__ void __launch_bounds__(1024) lse_push_kernel(const float *__restrict_
 }
 
 // Pass 2: every thread's column sums over its rows, added over the row threads at the tile's end.
-template <typename T, int D>
+// PAD: the rows end inside a tile of 64 (a kernel of its own: testing the rows costs whole tiles 1%,
+// and spares 32-row calls 1% of their exponentials).
+template <typename T, int D, bool PAD>
 __global__ void __launch_bounds__(kSimtThreads, 2) score_colsum_simt(
     const T *__restrict__ q_win, const T *__restrict__ K, const int32_t *__restrict__ lens, ScoreMask mask, int w, int G,
     int Hq, int Hkv, int L_cap, int R, int units, float c2, const float *__restrict__ rowb, float *__restrict__ raw,
@@ -344,7 +346,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) score_colsum_simt(
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const int r = r0 + ty + 16 * i;
-                        b[i] = r < R ? rowb[(long)run.u * R + r] : INFINITY;  // a padding row adds 2^-inf = 0
+                        b[i] = !PAD || r < R ? rowb[(long)run.u * R + r] : 0.f;
                     }
                     __syncthreads();  // the tiles before these have been read
                     if (r0 == 0) simt_load<T, D>(Ks, K + ((long)run.u * L_cap + j0) * D, kTile, nc - j0);
@@ -353,9 +355,12 @@ __global__ void __launch_bounds__(kSimtThreads, 2) score_colsum_simt(
                     float s[4][8];
                     simt_logits<D>(Qs, Ks, s);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j)
+                    for (int i = 0; i < 4; ++i) {
+                        // a padding row adds nothing, and its logit with an infinite key is NaN
+                        if (PAD && r0 + ty + 16 * i >= R) break;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) sum[j] += fast_exp2(fmaf(s[i][j], c2, -b[i]));
+                        for (int j = 0; j < 8; ++j) sum[j] += fast_exp2(fmaf(s[i][j], c2, -b[i]));
+                    }
                 }
                 __syncthreads();  // Qs has been read: the warps' sums go there
 #pragma unroll
@@ -543,9 +548,10 @@ static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *
                        units);
         if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    e = allow_smem((const void *)score_colsum_simt<T, D>, (int)smem);
+    auto colsum = R % kSimtRows ? score_colsum_simt<T, D, true> : score_colsum_simt<T, D, false>;
+    e = allow_smem((const void *)colsum, (int)smem);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(score_colsum_simt<T, D>, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap,
+    e = launch_pdl(colsum, grid, block, smem, s, q_win, K, lens, mask, w, G, kv.H_q, kv.H_kv, kv.L_cap,
                    R, (int)units, c2, (const float *)ws.rowb, ws.raw, mask.keep ? ws.ulist : nullptr,
                    mask.keep ? ws.ucount : nullptr);
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -75,3 +75,30 @@ def test_bf16_rows_beyond_the_tensor_cores():
     """R = 760 window rows at d = 64: the plain-FMA passes read bf16 rows."""
     wl = W.WORKLOADS["7b"].reduced(layers=1, batch=2, h_q=38, h_kv=2, d=64, L=700, decode_steps=0, w=40)
     _check(wl, np.array([[[700, 333], [40, 168]]], np.int32), 7, [(0, 0, 0), (0, 0, 1), (0, 1, 1)])
+
+
+@pytest.mark.parametrize("dtype,G,w,one_pass", [("f32", 1, 5, False), ("f32", 3, 32, False), ("f32", 3, 32, True),
+                                                ("f32", 2, 32, True), ("bf16", 19, 40, False)])
+def test_minus_infinity_in_a_key(dtype, G, w, one_pass):
+    """A key whose logit is -inf in every window row gets score 0 and changes no other score, also where
+    the rows end inside a 64-row tile: the same scores as with a finite element that underflows."""
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=1, h_q=2 * G, h_kv=2, d=64, L=300, decode_steps=0, w=w, dtype=dtype)
+    K, V = W.make_cache(wl, DEV, canary=False)
+    q = W.make_qwin(wl, DEV)
+    q[..., 0] = q[..., 0].abs() + 0.5
+    lens = torch.full((1, 1, 2), 300, dtype=torch.int32, device=DEV)
+    lse = torch.full((w, 1, 1, 2 * G), 6.0, dtype=torch.float32, device=DEV)
+    got = []
+    for x in (-float("inf"), -1e30):
+        K[0, 0, :, 20, 0] = x
+        if one_pass:
+            kv = reco.make_kv(K, V, wl.h_q)
+            scores = torch.zeros(K.shape[:4], dtype=torch.float32, device=DEV)
+            ws = reco.workspace(reco.RECO_OP_SCORE, kv, w, DEV)
+            reco.reco_score_cache_lse(kv, q, lens, lse, w, 1, wl.scale(), scores, ws)
+        else:
+            scores = gpu_score(wl, K, V, q, lens, 1)
+        reco.reco_check()
+        got.append(scores)
+    assert torch.all(got[0][0, 0, :, 20] == 0)
+    assert torch.equal(got[0], got[1])
