@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) score_rowstats_simt(
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     wait_prior_grid();  // lens, the queries and the cache may come from the previous kernels
     for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
-        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, false, part_tiles * kTile, skip, nullptr, nullptr, err);
+        n_runs = plan_runs<1>(plan, lens, mask, w, L_cap, units, false, part_tiles * kTile, skip, nullptr, nullptr, err);
         for (int e = 0; e < min(kPlanRuns, n_runs - skip); ++e) {
             const TileRun run = plan.run[e];
             const T *q = q_win + ((long)(run.u / Hkv) * Hq + (long)(run.u % Hkv) * G) * w * D;
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) score_colsum_simt(
     const float invG = 1.f / (float)G;
     wait_prior_grid();  // lens, the normalisers, the queries and the cache may come from the previous kernels
     for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
-        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, nullptr);
+        n_runs = plan_runs<1>(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, nullptr);
         for (int e = 0; e < min(kPlanRuns, n_runs - skip); ++e) {
             const TileRun run = plan.run[e];
             const int nc = run.L - w;
@@ -580,7 +580,7 @@ static cudaError_t score_simt_any(const reco_kv &kv, const void *q_win, const in
 }
 
 // Max-pooling of the raw scores into `scores`: over the unit list when the call built one
-// (a masked tensor-core call), else one CTA per (unit, tile of scores).
+// (a masked tensor-core call that was planned), else one CTA per (unit, tile of scores).
 static cudaError_t launch_pool(const reco_kv &kv, const int32_t *lens, ScoreMask mask, bool listed, int w, int pool,
                                float *scores, const ScoreWs &ws, cudaStream_t s)
 {
@@ -630,7 +630,7 @@ cudaError_t launch_score(const reco_kv &kv, const void *q_win, const int32_t *le
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, true);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, used_tc && keep, w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used_tc && keep && plan_items(units, kv.L_cap, kTile) > device_sm_count(), w, pool, scores, ws, s);
 }
 
 cudaError_t launch_lse_push(const float *lse, long n, float *ring, int slots, long long *slot, unsigned *err,
@@ -704,7 +704,7 @@ cudaError_t launch_score_lse(const reco_kv &kv, const void *q_win, const int32_t
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, false);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, used && keep, w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used && keep && plan_items(units, kv.L_cap, kTile) > device_sm_count(), w, pool, scores, ws, s);
 }
 
 }  // namespace reco

@@ -184,9 +184,14 @@ __device__ __forceinline__ bool elect_one()
 // pieces p = gt * MT + mt rotate through four TMEM regions of 128 columns.  A group of four
 // epilogue warps takes query tile mt of every EG-th key tile, whole: the groups work on
 // different regions and so drift apart, one exponentiating while another waits for its
-// accumulator, and a region is released by four warps.
-template <int D, int MT, int EG>
+// accumulator, and a region is released by four warps.  Where a unit has few tiles (SPLIT, for
+// caches of at most kSplitCap rows) that leaves groups idle and a tile's columns to one of them:
+// there every group takes its share of every tile's columns (4 units of 120 keys, both passes, 15.2 -> 14.2 us,
+// 160 of 500 keys 31.8 -> 30.4; 16384 keys 1.57 -> 1.61 ms).
+constexpr int kSplitCap = 1024;
+template <int D, int MT, int EG, bool SPLIT>
 struct Pass1Cfg {
+    static constexpr int CW = SPLIT ? kTile / EG : kTile;  // columns of a piece that a group takes
     static constexpr int HALVES = D / 64;
     static constexpr int BOX = kTile * 128;  // 128 rows x 128 bytes
     static constexpr int KSTAGE = HALVES * BOX;
@@ -251,16 +256,16 @@ template <int N> __device__ __forceinline__ float rowsum_tile(uint32_t ta, float
     return (a4[0] + a4[1]) + (a4[2] + a4[3]);
 }
 
-template <int D, int MT, int EG>
-__global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
+template <int D, int MT, int EG, bool SPLIT>
+__global__ void __launch_bounds__(Pass1Cfg<D, MT, EG, SPLIT>::THREADS, 1)
     score_rowstats_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const int32_t *__restrict__ lens, ScoreMask mask, int w, int G, int Hq, int Hkv, int L_cap, int R,
                       int n_chunks, int units, float c2, float *__restrict__ part_m, float *__restrict__ part_z,
                       unsigned *err)
 {
-    using C = Pass1Cfg<D, MT, EG>;
+    using C = Pass1Cfg<D, MT, EG, SPLIT>;
     constexpr int HALVES = C::HALVES, BOX = C::BOX, KSTAGE = C::KSTAGE;
-    constexpr int NR = C::NR, NS = C::NS, N = kTile;
+    constexpr int NR = C::NR, NS = C::NS, N = kTile, CW = C::CW;
     constexpr int CT = kScoreChunk / kTile;  // tiles per chunk
     constexpr uint32_t IDESC = idesc_bf16(128, N);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -286,7 +291,7 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
         }
         for (int b = 0; b < NR; ++b) {
             mbar_init(smem_addr(&bar_afull[b]), 1);
-            mbar_init(smem_addr(&bar_aempty[b]), 4);
+            mbar_init(smem_addr(&bar_aempty[b]), SPLIT ? 4 * EG : 4);
         }
         abort_sh = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -308,7 +313,7 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
     int gt = 0, nq = 0;  // tiles and query loads so far (each role counts its own)
     bool a_ready = false, k_ready = false;  // MMA issuer: the next piece's region, the next tile's keys
     for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
-        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, false, kScoreChunk, skip, nullptr, nullptr, err);
+        n_runs = plan_runs_call(plan, lens, mask, w, L_cap, units, false, kScoreChunk, skip, nullptr, nullptr, err);
         const int n_here = min(kPlanRuns, n_runs - skip);
         if (warp == 0) {  // producer: a unit's window queries, then its run's K tiles
             for (int e = 0; ok && e < n_here; ++e) {
@@ -382,7 +387,7 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
                     }
                 }
             }
-        } else {  // epilogue: query tile mt of every EG-th key tile, one window row per thread
+        } else {  // epilogue: query tile mt of every EG-th key tile (or CW columns of all), one window row per thread
             const int idx = (warp - 2) >> 2, mt = idx / EG, g = idx % EG, quarter = warp & 3;
             const int r = mt * 128 + quarter * 32 + lane;
             const bool warp_rows = mt * 128 + quarter * 32 < R;  // this warp holds real window rows
@@ -397,31 +402,32 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
                     // this group's tiles: every EG-th of the CTA's, so that it always meets its own TMEM
                     // regions.  They are every EG-th of the chunk's from its tile `first`: the partial goes
                     // by that, so a unit's partials do not depend on the plan
-                    const int first = (g - gt) & (EG - 1);
+                    const int first = SPLIT ? g : (g - gt) & (EG - 1), t0 = SPLIT ? c0 : c0 + first;
+                    const int col = SPLIT ? g * CW : 0;
                     float m = -INFINITY, z = 0.f;  // reference (log2 units) and sum relative to it
-                    for (int t = c0 + first; t < c1; t += EG) {
+                    for (int t = t0; t < c1; t += SPLIT ? 1 : EG) {
                         const int p = (gt + t - c0) * MT + mt, b = p % NR;
                         if (!(ok = warp_wait(smem_addr(&bar_afull[b]), (p / NR) & 1, abort_flag, err))) break;
                         tc_fence_after();
                         if (warp_rows) {
-                            const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * N);
-                            const int lim = min(j1 - 1, jmax) - t * N;  // columns 0..lim are visible
+                            const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * N + col);
+                            const int lim = min(j1 - 1, jmax) - t * N - col;  // columns 0..lim are visible
                             // a tile that every row sees whole is summed against the rows' references (at
                             // first the max of 16 columns) with no max pass; a masked tile, or a sum that
                             // could overflow (or is NaN), takes the rows' maxima, 16 columns at a time
                             bool summed = false;
-                            if (__all_sync(0xffffffffu, lim >= N - 1)) {
-                                if (t < c0 + EG) m = rowmax16(ta) * c2;
+                            if (__all_sync(0xffffffffu, lim >= CW - 1)) {
+                                if (t == t0) m = rowmax16(ta) * c2;
                                 if (__all_sync(0xffffffffu, m > -INFINITY)) {
-                                    const float sum = rowsum_tile<N>(ta, c2, m);
+                                    const float sum = rowsum_tile<CW>(ta, c2, m);
                                     summed = __all_sync(0xffffffffu, sum <= 0x1p96f);
                                     if (summed) z += sum;
                                 }
-                                if (!summed && t < c0 + EG) m = -INFINITY;
+                                if (!summed && t == t0) m = -INFINITY;
                             }
                             if (!summed) {
 #pragma unroll 1
-                                for (int k = 0; k < N / 16; ++k) {
+                                for (int k = 0; k < CW / 16; ++k) {
                                     float v[16];
                                     tmem_ld16_nowait(ta + 16 * k, v);
                                     tmem_ld_wait_regs<16>(v);
@@ -462,7 +468,12 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG>::THREADS, 1)
 // of a set splitting each piece's columns, one key per thread: the sets drift apart, so that one
 // exponentiates while the other waits.  A set must not meet a region whose piece before its own
 // may still be the other set's (the barrier's parity could not tell the two): with two chains and
-// only two regions (NQ > 320) all groups form one set.
+// only two regions (NQ > 320) all groups form one set.  So they do where every tile has a CTA of its
+// own (no second tile to drift to).
+// SHORT: calls of at most kShortTiles tiles per CTA, which a few us of planning would stretch, have the
+// plan inline and their barriers set by a warp: the trace's boundary takes 16.8 us, 19.1 otherwise;
+// long ones take 2% less without.
+constexpr int kShortTiles = 64;
 constexpr int kP2Groups = 4;
 constexpr int kP2Slots = 4;  // tiles whose other ranges' sums may wait for the first range's warps
 
@@ -513,7 +524,7 @@ __device__ __forceinline__ bool colsum_step(uint32_t &ta, const float *&b, int &
     return false;
 }
 
-template <int D>
+template <int D, bool SHORT>
 __global__ void __launch_bounds__(64 + 128 * kP2Groups, 1)
     score_colsum_tc(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                     const int32_t *__restrict__ lens, ScoreMask mask, int w, int G, int Hq, int Hkv, int L_cap, int R,
@@ -543,24 +554,31 @@ __global__ void __launch_bounds__(64 + 128 * kP2Groups, 1)
     const uint32_t Ks = base + HALVES * QBOXB;
     // per epilogue warp: the normalisers of its columns, after the K ring
     float *bsh = reinterpret_cast<float *>(smem_raw + (base - raw0) + HALVES * QBOXB + (size_t)NS * KSTAGE);
-    if (tid == 0) {
-        prefetch_tensormap(&tmQ);
-        prefetch_tensormap(&tmK);
-        mbar_init(smem_addr(&bar_qfull), 1);
-        mbar_init(smem_addr(&bar_qempty), 1);
-        for (int s = 0; s < NS; ++s) {
+    auto init_barriers = [&](int first, int step) {
+        if (first == 0) {
+            prefetch_tensormap(&tmQ);
+            prefetch_tensormap(&tmK);
+            mbar_init(smem_addr(&bar_qfull), 1);
+            mbar_init(smem_addr(&bar_qempty), 1);
+            abort_sh = 0;
+        }
+        for (int s = first; s < NS; s += step) {
             mbar_init(smem_addr(&bar_kfull[s]), 1);
             mbar_init(smem_addr(&bar_kempty[s]), 1);
         }
-        for (int b = 0; b < NR; ++b) {
+        for (int b = first; b < NR; b += step) {
             mbar_init(smem_addr(&bar_afull[b]), 1);
             mbar_init(smem_addr(&bar_aempty[b]), 4 * split);
         }
-        for (int k = 0; k < 4 * sets; ++k)
-            for (int sl = 0; sl < kP2Slots; ++sl) mbar_init(smem_addr(&bar_part[k][sl]), split - 1);
-        abort_sh = 0;
+        for (int k = first; k < 4 * sets * kP2Slots; k += step)
+            mbar_init(smem_addr(&bar_part[k / kP2Slots][k % kP2Slots]), split - 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_shared();
+    };
+    if constexpr (SHORT) {
+        if (warp == 0) init_barriers(lane, 32);
+    } else {
+        if (tid == 0) init_barriers(0, 1);
     }
     if (warp == 1) {
         tmem_alloc(smem_addr(&tmem_sh), kTmemCols);
@@ -586,8 +604,11 @@ __global__ void __launch_bounds__(64 + 128 * kP2Groups, 1)
     };
     for (int skip = 0, n_runs = 1; skip < n_runs; skip += kPlanRuns) {
         // with the normalisers given, this is the call's only pass: it reports lengths out of range
-        n_runs = plan_runs(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount,
-                           row_lse != nullptr ? err : nullptr);
+        unsigned *err_len = row_lse != nullptr ? err : nullptr;
+        if constexpr (SHORT)
+            n_runs = plan_runs<4>(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, err_len);
+        else
+            n_runs = plan_runs_call(plan, lens, mask, w, L_cap, units, true, kTile, skip, ulist, ucount, err_len);
         const int n_here = min(kPlanRuns, n_runs - skip);
         if (warp == 0) {  // producer
             const int qbox_rows = NQ > 256 ? NQ / 2 : NQ;
@@ -778,11 +799,11 @@ bool score_tc_supported(const reco_kv &kv, int w)
 // Pass-1 partials per chunk for R window rows (the combine merges them): the EG of pass1_by_mt.
 int score_tc_pass1_groups(int R) { return (R + 127) / 128 <= 2 ? 2 : 1; }
 
-template <int D, int MT, int EG>
+template <int D, int MT, int EG, bool SPLIT = false>
 static cudaError_t run_pass1(const reco_kv &kv, const void *q_win, const int32_t *lens, const ScoreMask &mask, int w,
                              float c2, const ScoreWs &ws, unsigned *err, cudaStream_t s, bool *ok)
 {
-    using C = Pass1Cfg<D, MT, EG>;
+    using C = Pass1Cfg<D, MT, EG, SPLIT>;
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
     const int R = (kv.H_q / kv.H_kv) * w;
     const int nch = (kv.L_cap + kScoreChunk - 1) / kScoreChunk;
@@ -793,10 +814,10 @@ static cudaError_t run_pass1(const reco_kv &kv, const void *q_win, const int32_t
         *ok = false;
         return cudaSuccess;
     }
-    cudaError_t e = allow_smem((const void *)score_rowstats_tc<D, MT, EG>, (int)C::SMEM);
+    cudaError_t e = allow_smem((const void *)score_rowstats_tc<D, MT, EG, SPLIT>, (int)C::SMEM);
     if (e != cudaSuccess) return e;
-    const int grid = (int)min(units * nch, (long)device_sm_count());
-    e = launch_pdl(score_rowstats_tc<D, MT, EG>, dim3(grid), dim3(C::THREADS), C::SMEM, s, mq, mk, lens, mask, w,
+    const int grid = (int)min(plan_items(units, kv.L_cap, kScoreChunk), (long long)device_sm_count());
+    e = launch_pdl(score_rowstats_tc<D, MT, EG, SPLIT>, dim3(grid), dim3(C::THREADS), C::SMEM, s, mq, mk, lens, mask, w,
                    kv.H_q / kv.H_kv, kv.H_q, kv.H_kv, kv.L_cap, R, nch, (int)units, c2, ws.part_m, ws.part_z, err);
     *ok = true;
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -807,6 +828,9 @@ static cudaError_t pass1_by_mt(const reco_kv &kv, const void *q_win, const int32
                                float c2, const ScoreWs &ws, unsigned *err, cudaStream_t s, bool *ok)
 {
     const int MT = ((kv.H_q / kv.H_kv) * w + 127) / 128;
+    if (kv.L_cap <= kSplitCap && MT <= 2)
+        return MT == 1 ? run_pass1<D, 1, 2, true>(kv, q_win, lens, mask, w, c2, ws, err, s, ok)
+                       : run_pass1<D, 2, 2, true>(kv, q_win, lens, mask, w, c2, ws, err, s, ok);
     switch (MT) {
     case 1: return run_pass1<D, 1, 2>(kv, q_win, lens, mask, w, c2, ws, err, s, ok);
     case 2: return run_pass1<D, 2, 2>(kv, q_win, lens, mask, w, c2, ws, err, s, ok);
@@ -840,7 +864,11 @@ static cudaError_t run_pass2(const reco_kv &kv, const void *q_win, const int32_t
         *ok = false;
         return cudaSuccess;
     }
-    const int sets = ps.NP + 1 <= ps.NR ? 2 : 1;  // (a set's pieces of consecutive turns lie NP + 1 apart)
+    const long long tiles = plan_items(units, kv.L_cap, kTile);
+    const int grid = (int)min(tiles, (long long)device_sm_count());
+    // two sets where they stay apart (a set's pieces of consecutive turns lie NP + 1 apart), and where a tile's
+    // columns are too few for all groups
+    const int sets = ps.NQ / ps.NP < 8 * kP2Groups || (ps.NP + 1 <= ps.NR && tiles > grid) ? 2 : 1;
     const size_t qbytes = (size_t)(D / 64) * ps.NQ * 128, kstage = (size_t)(D / 64) * kTile * 128;
     const size_t nbytes = (size_t)4 * sets * ps.NQ * sizeof(float);  // the epilogue warps' normalisers
     const size_t budget = 227 * 1024 - (sizeof(TilePlan) + 7 * 1024) - 1024;
@@ -850,12 +878,11 @@ static cudaError_t run_pass2(const reco_kv &kv, const void *q_win, const int32_t
     }
     const int NS = (int)min((size_t)4, (budget - qbytes - nbytes) / kstage);
     const size_t smem = 1024 + qbytes + (size_t)NS * kstage + nbytes;
-    cudaError_t e = allow_smem((const void *)score_colsum_tc<D>, (int)smem);
+    auto colsum = tiles <= (long long)kShortTiles * grid ? score_colsum_tc<D, true> : score_colsum_tc<D, false>;
+    cudaError_t e = allow_smem((const void *)colsum, (int)smem);
     if (e != cudaSuccess) return e;
-    const long tiles = units * ((kv.L_cap + kTile - 1) / kTile);
-    const int grid = (int)min(tiles, (long)device_sm_count());
     const bool masked = mask.keep != nullptr;
-    e = launch_pdl(score_colsum_tc<D>, dim3(grid), dim3(64 + 128 * kP2Groups), smem, s, mq, mk, lens, mask, w,
+    e = launch_pdl(colsum, dim3(grid), dim3(64 + 128 * kP2Groups), smem, s, mq, mk, lens, mask, w,
                    kv.H_q / kv.H_kv, kv.H_q, kv.H_kv, kv.L_cap, R, ps.NQ, ps.NP, ps.NR, NS, sets, (int)units, c2,
                    (const float *)ws.rowb, row_lse, (long)kv.n_layers * kv.B * kv.H_q, ws.raw,
                    masked ? ws.ulist : nullptr, masked ? ws.ucount : nullptr, err);

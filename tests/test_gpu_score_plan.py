@@ -102,3 +102,35 @@ def test_minus_infinity_in_a_key(dtype, G, w, one_pass):
         got.append(scores)
     assert torch.all(got[0][0, 0, :, 20] == 0)
     assert torch.equal(got[0], got[1])
+
+
+# short units: a CTA per item (few units), a planned call whose threads hold 1 to 4 units' lengths, more
+# units than that; one and two query tiles of split columns, three and two chains of whole tiles
+@pytest.mark.parametrize("layers,G,w,d,L", [(1, 4, 32, 128, 250), (1, 7, 32, 64, 1020), (2, 3, 16, 128, 120), (1, 10, 32, 128, 500),
+                                            (30, 8, 32, 128, 300), (160, 1, 5, 64, 140), (300, 2, 8, 64, 130),
+                                            (600, 1, 5, 64, 140), (30, 9, 32, 128, 200), (30, 5, 64, 128, 200)])
+def test_short_units(layers, G, w, d, L):
+    wl = W.WORKLOADS["7b"].reduced(layers=layers, batch=2, h_q=2 * G, h_kv=2, d=d, L=L, decode_steps=4, w=w)
+    rng = np.random.default_rng(layers + L)
+    lens = rng.integers(w, L + 1, (layers, 2, 2)).astype(np.int32)
+    lens[0, 0, 0], lens[0, 1, 1], lens[-1, 1, 0] = w, w + 1, L
+    units = [(0, 0, 0), (0, 1, 1), (layers - 1, 1, 0)] + [(int(rng.integers(layers)), b, h) for b in (0, 1) for h in (0, 1)]
+    _check(wl, lens, 5, units)
+    # one pass with given normalisers, sequence 1 masked out, in float64
+    K, V = W.make_cache(wl, DEV, canary=False)
+    q = W.make_qwin(wl, DEV)
+    kv = reco.make_kv(K, V, wl.h_q)
+    scores = torch.full(K.shape[:4], -1.0, dtype=torch.float32, device=DEV)
+    lse = torch.linspace(3.0, 6.0, w * layers * 2 * wl.h_q, device=DEV).view(w, layers, 2, wl.h_q)
+    keep = torch.tensor([0, 1 << 30], dtype=torch.int32, device=DEV)
+    reco.reco_score_cache_lse(kv, q, torch.from_numpy(lens).to(DEV), lse, w, 1, wl.scale(), scores,
+                              reco.workspace(reco.RECO_OP_SCORE, kv, w, DEV), keep=keep)
+    reco.reco_check()
+    assert torch.all(scores[:, 1] == -1.0)
+    for l, b, h in units:
+        if b == 1:
+            continue
+        n = int(lens[l, b, h]) - w
+        x = torch.einsum("gtd,jd->gtj", q[l, b, h * G:(h + 1) * G].double(), K[l, b, h, :n].double()) * wl.scale()
+        ref = torch.exp(x - lse[:, l, b, h * G:(h + 1) * G].double().T.unsqueeze(-1)).sum((0, 1)) / G
+        assert_scores_close(scores[l, b, h, :n].cpu().numpy(), ref.cpu().numpy(), f"unit {(l, b, h)}")
