@@ -392,6 +392,19 @@ __device__ __forceinline__ void pool_tile(const float *__restrict__ rp, int j0, 
 {
     constexpr int Q = kPoolTile / kPoolThreads / 4;  // groups of four consecutive scores per thread
     const int n = min(kPoolTile, nc - j0);
+    // at most a score per thread: straight from global memory, the window's loads in flight together (no
+    // shared memory, no barrier: 0.2 of 7.4 us for one pass over 4 units of 120 keys)
+    if (n <= kPoolThreads && half <= 4) {
+        const int j = j0 + (int)threadIdx.x;
+        if ((int)threadIdx.x < n) {
+            float m = __int_as_float(0x7fc00000);
+#pragma unroll
+            for (int o = -4; o <= 4; ++o)
+                if (o >= -half && o <= half && j + o >= 0 && j + o < nc) m = fmaxf(m, __ldcg(rp + j + o));
+            out[j] = m;
+        }
+        return;
+    }
     if (half > kPoolHalo) {
         for (int t = threadIdx.x; t < n; t += kPoolThreads) {
             const int j = j0 + t, lo = max(0, j - half), hi = min(nc - 1, j + half);
