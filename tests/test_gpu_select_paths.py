@@ -35,14 +35,19 @@ def _patterns(rng, n):
     ]
 
 
-SMS = 152
+def _sms():
+    return torch.cuda.get_device_properties(0).multi_processor_count
 
 
+# B sequences of two units each: a number, or (m, o) for m units per SM and o sequences more (the rules
+# have their lines at 1, 2, 4 and 6 units per SM)
 @pytest.mark.parametrize("B,most", [(16, m) for m in (1, 5, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000, 9001)]
-                         + [(B, m) for B in (SMS // 2, SMS // 2 + 1, SMS, SMS + 1) for m in (257, 1024, 1025)]
-                         + [(B, m) for B in (2 * SMS, 2 * SMS + 1, 3 * SMS, 3 * SMS + 1) for m in (257, 512, 513, 1024)]
-                         + [(2 * SMS + 1, 1025), (SMS, 16384), (SMS, 16385), (16, 40000)])
+                         + [(B, m) for B in ((1, 0), (1, 1), (2, 0), (2, 1)) for m in (257, 1024, 1025)]
+                         + [(B, m) for B in ((4, 0), (4, 1), (6, 0), (6, 1)) for m in (257, 512, 513, 1024)]
+                         + [((4, 1), 1025), ((2, 0), 16384), ((2, 0), 16385), (16, 40000)])
 def test_selection_by_length(B, most):
+    if isinstance(B, tuple):
+        B = B[0] * _sms() // 2 + B[1]
     rng = np.random.default_rng(most + 10007 * (B - 16))
     w = 5
     L_cap = most + w
