@@ -214,9 +214,13 @@ constexpr int kWholeBin = 0x7fffffff;
 // sweep, one scan of the warps' counts, one writing sweep.  The passes start below the bits that
 // all keys share (their smallest and largest key): scores of one unit lie within a few powers of
 // two, so a first digit of the top eight bits put nearly all keys into two or three bins, whose
-// atomics serialise.  Where there are more units than SMs, smaller CTAs share an SM and one counts
+// atomics serialise.  With few keys per thread (FEW: kFewKeys of them at most) that pass costs more than
+// it saves, and so do the sweeps as the compiler unrolls them for many: 112 units of 2056 rows 7.2 -> 6.0
+// us, of 8200 rows 11.5 -> 10.2; as for few, 1216 units of 16400 rows would take 99 instead of 81.
+// Where there are more units than SMs, smaller CTAs share an SM and one counts
 // while another waits at a barrier (512 units of 15000 to 16384 candidates: 54 -> 45 us).
-template <int NT>
+constexpr int kFewKeys = 8;  // keys per thread
+template <int NT, bool FEW>
 __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__ scores, const int32_t *lens,
                                                        int32_t *lens_out, const int32_t *__restrict__ keep, int w, int B, int Hkv,
                                                        int L_cap, int32_t *__restrict__ idx_out,
@@ -225,7 +229,7 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
     constexpr int NW = NT / 32;
     static_assert(NW <= 32, "one warp per lane of the warp-count scan");
     extern __shared__ uint32_t keys[];  // [L - w]
-    __shared__ int hist[256];
+    __shared__ __align__(16) int hist[256];
     __shared__ int w_gt[NW], w_eq[NW];
     __shared__ uint32_t w_min[NW], w_max[NW];
     __shared__ uint32_t s_prefix;
@@ -262,39 +266,50 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
             lo = min(lo, key);
             hi = max(hi, key);
         }
-        lo = __reduce_min_sync(0xffffffffu, lo);
-        hi = __reduce_max_sync(0xffffffffu, hi);
-        if (lane == 0) {
-            w_min[wid] = lo;
-            w_max[wid] = hi;
+        if constexpr (!FEW) {
+            lo = __reduce_min_sync(0xffffffffu, lo);
+            hi = __reduce_max_sync(0xffffffffu, hi);
+            if (lane == 0) {
+                w_min[wid] = lo;
+                w_max[wid] = hi;
+            }
+            __syncthreads();
+            lo = __reduce_min_sync(0xffffffffu, lane < NW ? w_min[lane] : 0xffffffffu);
+            hi = __reduce_max_sync(0xffffffffu, lane < NW ? w_max[lane] : 0u);
+        } else {  // (the search's barriers make the keys visible otherwise)
+            if (kc == 0) __syncthreads();
         }
-        __syncthreads();
-        lo = __reduce_min_sync(0xffffffffu, lane < NW ? w_min[lane] : 0xffffffffu);
-        hi = __reduce_max_sync(0xffffffffu, lane < NW ? w_max[lane] : 0u);
         uint32_t T = 0xffffffffu;
         int need = 0;
         if (kc > 0) {
-            int bits = 32 - __clz(lo ^ hi);  // the low bits in which keys differ
+            int bits = FEW ? 32 : 32 - __clz(lo ^ hi);  // the low bits in which keys (may) differ
             uint32_t prefix = bits < 32 ? hi >> bits << bits : 0u;
             uint32_t mask = bits < 32 ? ~0u << bits : 0u;
             int remaining = kc;
             while (bits > 0) {
                 const int shift = max(0, bits - 8);
-                for (int j = tid; j < nc; j += NT) {
-                    const uint32_t key = keys[j];
-                    // plain shared-memory atomics: grouping a warp's equal bins first
-                    // (__match_any_sync) cost more than the conflicts it saves
-                    if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
+                // plain shared-memory atomics: grouping a warp's equal bins first
+                // (__match_any_sync) cost more than the conflicts it saves
+                if constexpr (FEW) {
+                    for (int jb = 0; jb < nc; jb += NT) {
+                        const int j = jb + tid;
+                        const bool valid = j < nc;
+                        const uint32_t key = valid ? keys[j] : 0u;
+                        if (valid && (key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
+                    }
+                } else {
+                    for (int j = tid; j < nc; j += NT) {
+                        const uint32_t key = keys[j];
+                        if ((key & mask) == prefix) atomicAdd(&hist[(key >> shift) & 255u], 1);
+                    }
                 }
                 __syncthreads();
                 if (wid == 0) {  // find the bin holding the remaining-th largest key; clear for the next pass
-                    int c8[8], sum = 0;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        c8[i] = hist[255 - 8 * lane - i];
-                        hist[255 - 8 * lane - i] = 0;
-                        sum += c8[i];
-                    }
+                    int4 *h4 = reinterpret_cast<int4 *>(hist) + 62 - 2 * lane;  // bins 255 - 8 * lane and the seven below
+                    const int4 x = h4[1], y = h4[0];
+                    h4[0] = h4[1] = make_int4(0, 0, 0, 0);
+                    const int c8[8] = {x.w, x.z, x.y, x.x, y.w, y.z, y.y, y.x};
+                    const int sum = (x.x + x.y) + (x.z + x.w) + (y.x + y.y) + (y.z + y.w);
                     int incl = sum;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -329,13 +344,22 @@ __global__ void __launch_bounds__(NT) select_topm_smem(const float *__restrict__
         const int seg = (nc + NW - 1) / NW;
         const int j0 = min(nc, wid * seg), j1 = min(nc, j0 + seg);
         int n_gt = 0, n_eq = 0;
-        for (int j = j0 + lane; j < j1; j += 32) {
-            const uint32_t key = keys[j];
-            n_gt += key > T;
-            n_eq += key == T;
+        if constexpr (FEW) {
+            for (int jb = j0; jb < j1; jb += 32) {
+                const bool valid = jb + lane < j1;
+                const uint32_t key = valid ? keys[jb + lane] : 0u;
+                n_gt += __popc(__ballot_sync(0xffffffffu, valid && key > T));
+                n_eq += __popc(__ballot_sync(0xffffffffu, valid && key == T));
+            }
+        } else {
+            for (int j = j0 + lane; j < j1; j += 32) {
+                const uint32_t key = keys[j];
+                n_gt += key > T;
+                n_eq += key == T;
+            }
+            n_gt = __reduce_add_sync(0xffffffffu, n_gt);
+            n_eq = __reduce_add_sync(0xffffffffu, n_eq);
         }
-        n_gt = __reduce_add_sync(0xffffffffu, n_gt);
-        n_eq = __reduce_add_sync(0xffffffffu, n_eq);
         if (lane == 0) {
             w_gt[wid] = n_gt;
             w_eq[wid] = n_eq;
@@ -620,11 +644,11 @@ static cudaError_t launch_select_smem(const reco_kv &kv, size_t key_bytes, long 
                                       const int32_t *lens, int32_t *lens_out, const int32_t *keep, int w, int32_t *idx,
                                       int32_t *count, unsigned *err, cudaStream_t s)
 {
-    const cudaError_t e =
-        allow_smem((const void *)select_topm_smem<NT>, (int)kSelectSmemKeys * (int)sizeof(uint32_t));
+    auto fn = kv.L_cap - w <= kFewKeys * NT ? select_topm_smem<NT, true> : select_topm_smem<NT, false>;
+    const cudaError_t e = allow_smem((const void *)fn, (int)kSelectSmemKeys * (int)sizeof(uint32_t));
     if (e != cudaSuccess) return e;
-    return launch_pdl(select_topm_smem<NT>, dim3(walk_grid(select_topm_smem<NT>, NT, key_bytes, units, 1)), dim3(NT),
-                      key_bytes, s, scores, lens, lens_out, keep, w, kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
+    return launch_pdl(fn, dim3(walk_grid(fn, NT, key_bytes, units, 1)), dim3(NT), key_bytes, s, scores, lens, lens_out,
+                      keep, w, kv.B, kv.H_kv, kv.L_cap, idx, count, units, err);
 }
 
 static cudaError_t launch_select(const reco_kv &kv, const float *scores, const int32_t *lens, int32_t *lens_out,
@@ -652,14 +676,14 @@ static cudaError_t launch_select(const reco_kv &kv, const float *scores, const i
     if (key_bytes <= kSelectSmemKeys * sizeof(uint32_t)) {
         // Threads per unit, by how many units an SM can hold (as their keys allow) and has to: larger CTAs
         // are faster for one unit, smaller ones let one unit count while another waits at a barrier.  us with
-        // 256 / 512 / 1024 threads: 1 unit per SM of 4100 rows 10.9 / 8.9 / 7.7, of 1030 rows 6.9 / 5.8 / 6.3;
-        // 2 of 4100 rows 11.3 / 10.1 / 10.2; 3 of 16400 rows (1216 units) 79 / 65 / 72; 4 of 6200 rows
-        // 16.6 / 16.0 / 21.5; 8 of 4100 rows 22.6 / 24.4 / 33.1; 1216 units of 32800 rows, one per SM at a
-        // time, 383 / 211 / 157.
+        // 256 / 512 / 1024 threads: 1 unit per SM of 1544 rows 7.2 / 5.9 / 6.4, of 4104 rows 11.7 / 8.6 / 7.7;
+        // 2 of 4104 rows 12.1 / 10.0 / 10.9; 2 at a time of 20000 rows, 304 units 32.4 / 23.4 / 23.5, 608
+        // 73 / 47.5 / 46.4, 1216 147 / 93 / 88; 3 of 16400 rows (1216 units) 101 / 81 / 82; 4 of 4104 rows
+        // 13.7 / 15.4 / 19.5; 8 of 4104 rows 24.6 / 29 / 37.
         const long held = (long)((227 * 1024) / (key_bytes + 4096)), per_sm = std::min((units + sms - 1) / sms, held);
         if ((per_sm <= 1 && most > 2048) || (per_sm == 2 && most > 16 * 1024))
             e = launch_select_smem<1024>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
-        else if (per_sm <= 4)
+        else if (per_sm <= 3)
             e = launch_select_smem<512>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);
         else
             e = launch_select_smem<256>(kv, key_bytes, units, scores, lens, lens_out, keep, w, idx, count, err, s);

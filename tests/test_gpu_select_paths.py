@@ -40,11 +40,13 @@ def _sms():
 
 
 # B sequences of two units each: a number, or (m, o) for m units per SM and o sequences more (the rules
-# have their lines at 1, 2, 4 and 6 units per SM)
+# have their lines at 1, 2, 3, 4 and 6 units per SM)
 @pytest.mark.parametrize("B,most", [(16, m) for m in (1, 5, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 3000, 9001)]
                          + [(B, m) for B in ((1, 0), (1, 1), (2, 0), (2, 1)) for m in (257, 1024, 1025)]
-                         + [(B, m) for B in ((4, 0), (4, 1), (6, 0), (6, 1)) for m in (257, 512, 513, 1024)]
-                         + [((4, 1), 1025), ((2, 0), 16384), ((2, 0), 16385), (16, 40000)])
+                         + [(B, m) for B in ((3, 0), (3, 1), (4, 0), (4, 1), (6, 0), (6, 1)) for m in (257, 512, 513, 1024)]
+                         + [((4, 1), 1025), ((2, 0), 16384), ((2, 0), 16385), (16, 40000)]
+                         # eight keys per thread and one more, with 1024, 512 and 256 threads
+                         + [(16, 8192), (16, 8193), ((3, 0), 4096), ((3, 0), 4097), ((6, 0), 2048), ((6, 0), 2049)])
 def test_selection_by_length(B, most):
     if isinstance(B, tuple):
         B = B[0] * _sms() // 2 + B[1]
