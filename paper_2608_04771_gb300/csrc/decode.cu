@@ -555,6 +555,7 @@ template <int D_, int GT_> struct F32Block {
     static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = KB * GT;
     static constexpr bool TENSOR_MAPS = false;
     static constexpr bool DEEP = false;  // bound by its arithmetic: all the warps (93 against 70 us)
+    static constexpr int GP = GT == 8 ? 4 : GT;  // heads per turn of the PV product
     static constexpr int VPL = GT == 8 ? 2 : (GT == 6 ? 3 : 1);  // (key, head) sums per lane
 
     float q[GT][QE], o[GT][E], m[VPL], l[VPL];
@@ -695,41 +696,53 @@ template <int D_, int GT_> struct F32Block {
             p_sm[kk * GT + head_of(v)] = p;
         }
         __syncwarp();
+        // A block's products are summed before they are added to the output: the chain of additions into it
+        // is as long as the item's blocks, not its keys.  Eight heads take the block in two turns
+        // (registers).
 #pragma unroll
-        for (int k = 0; k < KB; ++k) {
-            float p[GT], x[E];
-            if constexpr (GT % 4 == 0) {
+        for (int g0 = 0; g0 < GT; g0 += GP) {
+            if (g0 > 0) __syncwarp();
+            float acc[GP][E];
 #pragma unroll
-                for (int g = 0; g < GT; g += 4) {
-                    const float4 f = *reinterpret_cast<const float4 *>(p_sm + k * GT + g);
-                    p[g] = f.x;
-                    p[g + 1] = f.y;
-                    p[g + 2] = f.z;
-                    p[g + 3] = f.w;
+            for (int k = 0; k < KB; ++k) {
+                float p[GP], x[E];
+                if constexpr (GP % 4 == 0) {
+#pragma unroll
+                    for (int g = 0; g < GP; g += 4) {
+                        const float4 f = *reinterpret_cast<const float4 *>(p_sm + k * GT + g0 + g);
+                        p[g] = f.x;
+                        p[g + 1] = f.y;
+                        p[g + 2] = f.z;
+                        p[g + 3] = f.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int g = 0; g < GP; g += 2) {
+                        const float2 f = *reinterpret_cast<const float2 *>(p_sm + k * GT + g0 + g);
+                        p[g] = f.x;
+                        p[g + 1] = f.y;
+                    }
                 }
-            } else {
-#pragma unroll
-                for (int g = 0; g < GT; g += 2) {
-                    const float2 f = *reinterpret_cast<const float2 *>(p_sm + k * GT + g);
-                    p[g] = f.x;
-                    p[g + 1] = f.y;
+                if constexpr (E == 4) {
+                    const float4 f = lds_f4(Vs + k * ROW + lane * 16);
+                    x[0] = f.x;
+                    x[1] = f.y;
+                    x[2] = f.z;
+                    x[3] = f.w;
+                } else {
+                    const float2 f = lds_f2(Vs + k * ROW + lane * 8);
+                    x[0] = f.x;
+                    x[1] = f.y;
                 }
-            }
-            if constexpr (E == 4) {
-                const float4 f = lds_f4(Vs + k * ROW + lane * 16);
-                x[0] = f.x;
-                x[1] = f.y;
-                x[2] = f.z;
-                x[3] = f.w;
-            } else {
-                const float2 f = lds_f2(Vs + k * ROW + lane * 8);
-                x[0] = f.x;
-                x[1] = f.y;
+#pragma unroll
+                for (int g = 0; g < GP; ++g)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) acc[g][e] = k ? fmaf(p[g], x[e], acc[g][e]) : p[g] * x[e];
             }
 #pragma unroll
-            for (int g = 0; g < GT; ++g)
+            for (int g = 0; g < GP; ++g)
 #pragma unroll
-                for (int e = 0; e < E; ++e) o[g][e] = fmaf(p[g], x[e], o[g][e]);
+                for (int e = 0; e < E; ++e) o[g0 + g][e] += acc[g][e];
         }
     }
 

@@ -113,3 +113,24 @@ def test_rings():
         assert torch.equal(out, ref_o) and torch.equal(lens, ref_l)
         assert torch.equal(ring[s], ref_lse.flatten()) and torch.equal(ring[s + S], ref_lse.flatten())
         assert torch.equal(q_ring[..., s, :], q) and int(slot) == (s + 1) % S
+
+
+def test_rounding_does_not_grow_with_the_keys():
+    """Errors against float64. An output is a sum of about n = 720 random terms in one warp: added one by one,
+    each rounding (2^-24 / sqrt(3) of the partial sum on average over its binade) would give
+    1.7e-8 * sqrt(n / 2) = 3.2e-7 of the result, blocks of 8 first 1.1e-7; the exponentials and logits add
+    about 2e-7 in either case."""
+    wl = _wl(8, 4, 128, 1155, layers=12, batch=21, steps=1)
+    lens_np = np.random.default_rng(5).integers(577, 1156, (12, 21, 4)).astype(np.int32)
+    K, V = W.make_cache(wl, DEV, canary=False)
+    q, _, _ = W.make_decode_step(wl, 0, DEV)
+    out, _ = gpu_decode(wl, K, V, torch.from_numpy(lens_np).to(DEV), q)
+    reco.reco_check()
+    num = den = 0.0
+    for l, b, h in [(l, b, h) for l in range(0, 12, 3) for b in range(0, 21, 5) for h in range(4)]:
+        n, hq = int(lens_np[l, b, h]), slice(8 * h, 8 * h + 8)
+        p = torch.softmax(q[l, b, hq].double() @ K[l, b, h, :n].double().T * wl.scale(), 1)
+        ref = p @ V[l, b, h, :n].double()
+        num += float((out[l, b, hq].double() - ref).square().sum())
+        den += float(ref.square().sum())
+    assert (num / den) ** 0.5 < 3e-7
