@@ -271,6 +271,7 @@ constexpr int kMaxTmaUnits = 8192;    // one plan entry per unit kept in shared 
 constexpr long long kSpinLimit = 1LL << 24;  // bounded mbarrier waits (about a second)
 constexpr float kLazyLog2 = 8.f;             // output rescale threshold (log2 units)
 constexpr int kMinBlocksPerWarp = 4;         // fewer working warps rather than shorter ranges
+constexpr int kCheapPieces = 8;              // pieces of a unit that are merged without a thought
 constexpr int kMaxWholeBlocks = 16;          // units of at most this many blocks are never cut
 constexpr int kOnePassBlocks = 16;           // blocks per warp from which all heads of a unit run in one pass
 constexpr int kDeepBlocksPerWarp = 64;       // from this many blocks per warp, half the warps with deep rings
@@ -982,19 +983,30 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         __syncthreads();
     }
     bool aborted = false;
+    // Working warps W: every one gets at least kMinBlocksPerWarp blocks (or all warps work), and no unit is
+    // cut into too many pieces: one warp merges a unit's pieces one after another, each at about the cost
+    // of (GS + 1) / 8 blocks.  With NB / W blocks per warp and max_nb * W / NB pieces of the longest unit, the
+    // one time falls as the other grows; they are about equal at W^2 = 8 NB^2 / (max_nb (GS + 1)).  Up to
+    // kCheapPieces pieces the merge costs less than the idle warps would.  us on all warps and so: 2 units
+    // of 32000 rows, 7 heads 358 and 65; one such unit among 200 of 16 rows 372 and 75, among 15 of 900
+    // rows 361 and 65.  Units of one length are cut into one number of pieces, unless that leaves warps idle that
+    // have 8 blocks or more to do: then no warp has two pieces, of which each costs it a publication (some
+    // 5 us: 8 units of 500 rows 20.8 on 45 warps, 18.2 on 64; 200 of 763 rows, 7 heads, 32.8 on 1216, 27.5 on
+    // 1200; 224 units of 1500 rows, 44 blocks a warp, are bound by their bytes on either).
+    const int all_warps = (deep ? NW / 2 : NW) * (int)gridDim.x;
+    int W = max(1, min(all_warps, NB / kMinBlocksPerWarp));
+    if (!snake) {  // (in floats: 64-bit products and divisions here cost a short call 0.2 to 0.5 us)
+        const float fb = (float)NB;
+        if ((float)max_nb * (float)W > kCheapPieces * fb)
+            W = max(1, min(W, (int)(fb * rsqrtf(0.125f * (float)max_nb * (float)(GS + 1)))));
+        if ((W < all_warps || NB < 8 * all_warps) && W >= n_ne && n_ne > 0 && NB - max_nb * n_ne == 0) W -= W % n_ne;
+    }
     // the warp's items, by block consumer C
     auto run = [&](auto tag) {
     using C = typename decltype(tag)::type;
     constexpr int GM = C::GM;
     const int NWm = deep ? NW / 2 : NW, Sm = deep ? 2 * S : S;  // NWm * Sm == NW * S either way
     const uint32_t my_ring = ring0 + (uint32_t)wid * Sm * STAGE;
-    // Working warps: every one gets at least kMinBlocksPerWarp blocks (or all warps work), and few
-    // units are cut into few pieces: one warp merges a unit's pieces one after another, each at about
-    // the cost of a block, so pieces per unit do not exceed blocks per warp, W^2 <= NB * units
-    // (2 units of 32000 rows, 7 heads: 341 us on all warps, 74 so, 100 with sqrt(5) times as many;
-    // from some 40 long units on every warp works).
-    int W = max(1, min(NWm * (int)gridDim.x, NB / kMinBlocksPerWarp));
-    while (W > 1 && (long long)W * W > (long long)NB * n_ne) W -= max(1, W >> 4);
     const bool out_bf16 = a.out_bf16 != 0;
     auto wstart = [&](int w) { return (int)((long long)w * NB / W); };  // ideal first block of warp w
     auto owner = [&](int b) { return (int)(((long long)(b + 1) * W - 1) / NB); };  // ideal owner of block b

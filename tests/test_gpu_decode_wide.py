@@ -58,3 +58,30 @@ def test_few_units(units, G, L):
     wl = W.WORKLOADS["7b"].reduced(layers=1, batch=units, h_q=G, h_kv=1, L=L, decode_steps=1)
     lens = np.random.default_rng(L).integers(L // 2, L + 1, (1, units, 1)).astype(np.int32)
     _check(wl, lens, [(0, 0, 0), (0, units - 1, 0)])
+
+
+# a long unit among short ones: it is cut into as many pieces as balance its merge, whatever the
+# number of short units (never cut) beside it
+@pytest.mark.parametrize("short,G,L", [(1, 7, 20000), (40, 4, 32000), (600, 7, 32000), (63, 16, 9000)])
+def test_one_long_unit_among_short_ones(short, G, L):
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=short + 1, h_q=G, h_kv=1, L=L, decode_steps=1)
+    lens = np.random.default_rng(L).integers(1, 250, (1, short + 1, 1)).astype(np.int32)
+    long = short // 2
+    lens[0, long, 0] = L
+    _check(wl, lens, [(0, 0, 0), (0, long, 0), (0, short, 0)])
+
+
+# units of one length: whole numbers of pieces, also where the cap or the blocks per warp leave a remainder
+@pytest.mark.parametrize("units,G,L", [(8, 7, 500), (7, 1, 763), (31, 4, 1500), (3, 16, 9000), (150, 8, 763)])
+def test_units_of_one_length(units, G, L):
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=units, h_q=G, h_kv=1, L=L, decode_steps=1)
+    _check(wl, np.full((1, units, 1), L - 1, np.int32), [(0, 0, 0), (0, units // 2, 0), (0, units - 1, 0)])
+
+
+def test_no_unit_with_keys():
+    wl = W.WORKLOADS["7b"].reduced(layers=1, batch=3, h_q=2, h_kv=1, L=64, decode_steps=1)
+    K, V = W.make_cache(wl, DEV, canary=False)
+    q, _, _ = W.make_decode_step(wl, 0, DEV)
+    out, lse = gpu_decode(wl, K, V, torch.zeros((1, 3, 1), dtype=torch.int32, device=DEV), q)
+    reco.reco_check()
+    assert torch.all(out == 0) and torch.all(torch.isneginf(lse))

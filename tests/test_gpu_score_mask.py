@@ -85,6 +85,15 @@ def test_fp32_mask_simt_path():
     assert _check(wl, lens, keep) == 2 * 2 * wl.h_kv
 
 
+def test_fp32_mask_few_sequences_several_pool_tiles():
+    """One sequence of twelve scored, its units longer than a pooling tile (4096 scores)."""
+    wl = W.WORKLOADS["tiny"].reduced(layers=2, batch=12, L=4500, decode_steps=0)
+    lens = np.random.default_rng(14).integers(4200, wl.L_cap + 1, (2, 12, wl.h_kv)).astype(np.int32)
+    keep = np.full(12, 1 << 30, np.int32)
+    keep[7] = wl.w
+    assert _check(wl, lens, keep) == 2 * 11 * wl.h_kv
+
+
 def test_mask_that_skips_everything_and_nothing():
     wl = W.WORKLOADS["7b"].reduced(layers=1, batch=3, L=900, decode_steps=10)
     lens = _ragged(wl, 13)
