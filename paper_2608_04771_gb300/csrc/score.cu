@@ -536,6 +536,9 @@ cudaError_t launch_score_tc_pass2(const reco_kv &kv, const void *q_win, const in
                                   cudaStream_t s, bool *used);
 int score_tc_pass1_groups(int R);
 
+// CTAs of a column-sum pass: one per SM on the tensor cores, two on plain FMAs.
+static long colsum_ctas(bool tc) { return (tc ? 1L : 2L) * device_sm_count(); }
+
 // Passes on plain FMAs; with pass1 false the row normalisers are already in ws.rowb.  A masked
 // call's pass 2 also lists the units it scored in ws.ulist / ws.ucount.
 template <typename T, int D>
@@ -545,7 +548,7 @@ static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
     const int G = kv.H_q / kv.H_kv, R = G * w;
     const long tiles = units * ((kv.L_cap + kTile - 1) / kTile);
-    const dim3 grid((unsigned)std::min(tiles, 2L * device_sm_count())), block(kSimtThreads);
+    const dim3 grid((unsigned)std::min(tiles, colsum_ctas(false))), block(kSimtThreads);
     constexpr size_t smem = SimtSmem<D>::BYTES;
     const T *K = (const T *)kv.k;
     cudaError_t e = cudaSuccess;
@@ -592,14 +595,15 @@ static cudaError_t score_simt_any(const reco_kv &kv, const void *q_win, const in
                                                 pass1);
 }
 
-// Max-pooling of the raw scores into `scores`: over the unit list when the call built one
-// (a masked tensor-core call that was planned), else one CTA per (unit, tile of scores).
-static cudaError_t launch_pool(const reco_kv &kv, const int32_t *lens, ScoreMask mask, bool listed, int w, int pool,
+// Max-pooling of the raw scores into `scores`: over the unit list where the column sums (on the tensor
+// cores, or not) built one, which a masked call's do unless every item has its CTA; else one CTA per
+// (unit, tile of scores).
+static cudaError_t launch_pool(const reco_kv &kv, const int32_t *lens, ScoreMask mask, bool tc, int w, int pool,
                                float *scores, const ScoreWs &ws, cudaStream_t s)
 {
     const long units = (long)kv.n_layers * kv.B * kv.H_kv;
     const unsigned chunks = (unsigned)((kv.L_cap + kPoolTile - 1) / kPoolTile);
-    if (listed) {
+    if (mask.keep != nullptr && plan_items(units, kv.L_cap, kTile) > colsum_ctas(tc)) {
         const long walkers = std::max(1L, 8L * device_sm_count() / (long)chunks);
         const unsigned ys = (unsigned)std::min(units, std::min(walkers, 65535L));
         cudaError_t e = launch_pdl(score_pool_list, dim3(chunks, ys), dim3(kPoolThreads), 0, s, (const float *)ws.raw, lens,
@@ -643,7 +647,7 @@ cudaError_t launch_score(const reco_kv &kv, const void *q_win, const int32_t *le
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, true);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, used_tc && keep && plan_items(units, kv.L_cap, kTile) > device_sm_count(), w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used_tc, w, pool, scores, ws, s);
 }
 
 cudaError_t launch_lse_push(const float *lse, long n, float *ring, int slots, long long *slot, unsigned *err,
@@ -717,7 +721,7 @@ cudaError_t launch_score_lse(const reco_kv &kv, const void *q_win, const int32_t
         e = score_simt_any(kv, q_win, lens, mask, w, c2, ws, err, s, false);
         if (e != cudaSuccess) return e;
     }
-    return launch_pool(kv, lens, mask, used && keep && plan_items(units, kv.L_cap, kTile) > device_sm_count(), w, pool, scores, ws, s);
+    return launch_pool(kv, lens, mask, used, w, pool, scores, ws, s);
 }
 
 }  // namespace reco
