@@ -16,10 +16,10 @@
 //   and PV on mma.sync m16n8k16 (fp32 accumulate), up to 16 query heads.  The head
 //   dimension is permuted consistently on the Q and K sides (and on the V and output
 //   sides) so that each thread's fragments are whole 16-byte chunks, and the swizzle makes
-//   every fragment read conflict-free.  Heads 9 to 16 of a unit fill the QK tile's other
-//   eight rows: one pass over the block instead of two units of half the heads (28 x 4 x 4
-//   units of 2000 to 4100 rows, 16 heads: 217 -> 145 us).  Where a warp would get under 16
-//   blocks so, the halves stay units of their own.
+//   every fragment read conflict-free.  A unit of 9 to 16 heads runs as two units of half the
+//   heads (28 x 4 x 4 units of 2000 to 4100 rows, 16 heads: 215 -> 128 us from half the warps
+//   with deep rings to all of them); with many short units its other heads fill the QK tile's
+//   other eight rows instead, one pass over the block.
 //   float32: blocks of 8 keys, plain FMAs (28 x 4 x 2 units of 800 to 1500 rows, 6 heads,
 //   from one CTA per unit that took its keys one by one: 514 -> 60 us).
 // A unit split over several items writes partial (max, sum, output) triples; the last
@@ -273,7 +273,9 @@ constexpr float kLazyLog2 = 8.f;             // output rescale threshold (log2 u
 constexpr int kMinBlocksPerWarp = 4;         // fewer working warps rather than shorter ranges
 constexpr int kCheapPieces = 8;              // pieces of a unit that are merged without a thought
 constexpr int kMaxWholeBlocks = 16;          // units of at most this many blocks are never cut
-constexpr int kOnePassBlocks = 16;           // blocks per warp from which all heads of a unit run in one pass
+constexpr int kOnePassBlocks = 16;           // blocks per warp from which all heads of a unit may run in one pass
+// units from which they may, of `warps` warps
+__host__ __device__ constexpr int one_pass_units(int warps) { return warps * 2 / 3; }
 constexpr int kDeepBlocksPerWarp = 64;       // from this many blocks per warp, half the warps with deep rings
 
 constexpr int kStageBytes128 = 8192;         // a block of K and V rows at d = 128 (half of it at d = 64)
@@ -319,8 +321,8 @@ template <int D_, int NT_, int HALVES_ = 1> struct Bf16Block {
     static constexpr int ROW = 2 * D, HALVES = D / 64, TILE = 16 * 128, MT = D / 16;
     static constexpr int APP = (2 * ROW / 16 + 31) / 32, SCRATCH = 0;
     static constexpr bool TENSOR_MAPS = true, PREFETCH_Q = NT == 1;
-    // half the warps with deeper rings for long work: up to eight heads a block leaves a warp
-    // waiting for data; with more its arithmetic wants all the warps (160 against 155 us)
+    // half the warps with deeper rings for long work: with up to eight heads a block leaves a warp
+    // waiting for data
     static constexpr bool DEEP = true;
 
     uint32_t qa[D / 16][2 * NT], qn[PREFETCH_Q ? D / 16 : 1][2 * NT];
@@ -905,12 +907,15 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
         n_ne += sm_red[NW + w2];
     }
     // Units of more than 8 query heads may run as two virtual units of half the heads over the same
-    // rows (float32 always does).  One pass over a block for all heads costs less than two when the
-    // warps are busy with blocks; with few blocks per warp, twice as many units keep more warps busy
-    // and their merges are half as large.  Measured (one pass against halves, us): 448 units of 2000
-    // to 4100 rows 142 : 217, 1456 of 187 to 750 80 : 116, 648 of 328 44 : 41, 450 of 272 to 818
-    // 54 : 47, 198 of 525 46 : 37, 8 of 12000 to 24000 331 : 84.
-    const int hs = !Block::SPLIT ? 1 : (Block::ALWAYS ? 2 : (pb[P] >= kOnePassBlocks * total_warps ? a.hs_min : a.hs_max));
+    // rows (float32 always does): twice as many units keep more warps busy, their merges are half as
+    // large, and the second read of a row mostly hits L2.  One pass for all heads is faster only with
+    // many short units (few cuts) and many blocks per warp.  One pass : halves, us, 9 and 16 heads:
+    // 1792 units of 225 to 300 rows 63 : 70 and 68 : 70, 896 of 375 to 500 51 : 55 and 57 : 57, of 600 to 800
+    // 70 : 73 and 76 : 75; but 448 of 750 to 1000 57 : 51 and 65 : 53, of 2000 to 4100 142 : 128 (16 heads), 224
+    // of 2250 to 3000 81 : 66 and 88 : 68, 64 of 6000 to 8000 91 : 58 and 96 : 62, 896 of 150 to 200 30 : 29 and
+    // 30 : 29.
+    const bool one_pass = P >= one_pass_units(total_warps) && pb[P] >= kOnePassBlocks * total_warps;
+    const int hs = !Block::SPLIT ? 1 : (Block::ALWAYS ? 2 : (one_pass ? a.hs_min : a.hs_max));
     // Virtual unit u covers half u / P (of gv heads) of the cache unit u % P: all first halves come
     // first in the plan, then all second halves in the same order, so warps w and w + W/2 stream
     // the same rows at about the same time and the second read mostly hits L2.
@@ -936,7 +941,10 @@ __global__ void __launch_bounds__(kDecodeWarps * 32, 1)
     // Fewer than half as many units as warps (with at least 8 blocks per warp) also
     // takes the deep partition: there the 8-warp split would cut every unit into many
     // pieces, whose merges cost more than the shallower rings save.
-    const bool deep = Block::DEEP && GS <= 8 && (NB >= kDeepBlocksPerWarp * total_warps ||
+    // Not halves: their second read comes from L2, so warps wait less for data and more for each other
+    // (448 units of 2000 to 4100 rows, 16 heads, 215 us on half the warps, 128 on all; 224 of 1500 to 2000 74
+    // and 53).
+    const bool deep = Block::DEEP && hs == 1 && GS <= 8 && (NB >= kDeepBlocksPerWarp * total_warps ||
                                       (NB >= 8 * total_warps && total_warps > 2 * units));
     // Only short units (none is ever cut): the contiguous deal below would leave some warps
     // two whole units where others have one.  Instead the units are sorted by blocks, most
@@ -1543,10 +1551,12 @@ cudaError_t launch_decode(const reco_kv &kv, const void *q, const void *k_new, c
         const int gt = a.G > 6 ? 8 : (a.G + 1) / 2 * 2;  // (halves of more than 8 heads: by the widest)
         fn = kv.d == 64 ? f32_kernel<64>(gt) : f32_kernel<128>(gt);
     } else {
-        // With more than 8 heads: a cache that cannot hold 24 blocks a warp runs as halves in any case
-        // (the kernel of one consumer is up to 10% faster there than the one that may choose).
+        // With more than 8 heads: calls that run as halves in any case, as few units or a cache that cannot
+        // hold 24 blocks a warp tell, take the kernel of one consumer (64 units of 6000 to 8000 rows, 16
+        // heads, 62 us against 69 in the kernel that may choose, 448 of 750 to 1000 53 against 58).
+        const int warps = kDecodeWarps * device_sm_count();
         const bool halves = a.G > 8 && 2LL * std::min<long long>(a.units, kMaxTmaUnits) <= kMaxTmaUnits &&
-                            (long long)a.units * ((kv.L_cap + 15) / 16) < 24LL * kDecodeWarps * device_sm_count();
+                            (a.units < one_pass_units(warps) || (long long)a.units * ((kv.L_cap + 15) / 16) < 24LL * warps);
         fn = kv.d == 64 ? bf16_kernel<64>(a.G > 8, halves) : bf16_kernel<128>(a.G > 8, halves);
     }
     // More units than one plan holds in shared memory run as consecutive launches over
