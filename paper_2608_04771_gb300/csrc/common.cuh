@@ -59,8 +59,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 
 // Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The largest size
 // asked for is remembered per kernel and device (a kernel is known by its function, which never
-// goes away), so that most calls set no attribute: the Tiny step of eleven launches, bound by the
-// host, went from 107 to 92 us with this and plain integers for pointers in the binding.
+// goes away; the runtime sets the limit again in a new context of the device and after a device
+// reset), so that most calls set no attribute, and calls from several threads never lower each
+// other's: the Tiny step of eleven launches, bound by the host, went from 107 to 92 us with this
+// and plain integers for pointers in the binding.
 cudaError_t allow_smem(const void *kernel, int bytes);
 
 // 2^x on the MUFU pipe (ex2.approx.ftz.f32).

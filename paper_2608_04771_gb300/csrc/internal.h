@@ -21,10 +21,11 @@ constexpr int kSampleMaxSeg = 1024;
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct ScoreWs {  // regions carved from the caller's workspace
-    float *part_m, *part_z;  // [units][n_chunks][R]  per-chunk row max (log2) / row sum
+    float *part_m, *part_z;  // [units][parts][R]     a part's row reference (log2) / row sum: up to two parts per 2048
+                             // keys on the tensor cores, one per 128 keys otherwise
     float *rowb;             // [units][R]            log2 of the row normaliser
     float *raw;              // [units][L_cap]        unpooled scores
-    int32_t *ulist;          // [units]               units to score, ascending (with a keep mask)
+    int32_t *ulist;          // [units]               units scored by a planned masked call, ascending
     int32_t *ucount;         // [1]                   entries of ulist
     size_t bytes;
 };
@@ -52,7 +53,8 @@ struct SelectWs {
 };
 
 struct DecodeWs {
-    int32_t *counters;  // [2 + units]: [0] a warp stopped early, [1] finished warps, [2 + u] merge tickets
+    int32_t *counters;  // [2 + units], or [2 + 2 * units] for G > 8: [0] warps stopped early, [1] finished warps,
+                        // [2 + u] merge tickets (of halves: [2 + units + u] too)
     float *part_ml;     // [part_slots][G][2]  (m log2, l)
     float *part_o;      // [part_slots][G][d]  unnormalised output
     int part_slots;

@@ -573,7 +573,9 @@ static cudaError_t score_simt(const reco_kv &kv, const T *q_win, const int32_t *
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Largest R*D (and R more) the calls outside the tensor-core passes accept.
+// Largest R*D (and R more) the calls outside the tensor-core passes accept: the shapes that fitted an
+// earlier kernel, which held all of a unit's window queries in shared memory.  These passes need no
+// limit; it stays as the interface's, with which callers choose their windows.
 constexpr size_t kSimtMaxQ = 200 * 1024 / 4;
 
 bool score_shape_supported(const reco_kv &kv, int w)
