@@ -21,7 +21,7 @@
 //   with deep rings to all of them); with many short units its other heads fill the QK tile's
 //   other eight rows instead, one pass over the block.
 //   float32: blocks of 8 keys, plain FMAs (28 x 4 x 2 units of 800 to 1500 rows, 6 heads,
-//   from one CTA per unit that took its keys one by one: 514 -> 60 us).
+//   from one CTA per unit that took its keys one by one: 540 -> 61 us).
 // A unit split over several items writes partial (max, sum, output) triples; the last
 // item to finish (atomic ticket, no waiting) merges them.  The counters live in the
 // caller's workspace, zero-filled before its first use; each launch clears what it

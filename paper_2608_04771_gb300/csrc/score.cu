@@ -65,9 +65,10 @@ ScoreWs score_ws_layout(const reco_kv &kv, int w, void *base)
 // while the other multiplies, share the call's tiles as the plan deals them.
 //
 // The FMA issue bounds it: a thread's 128 FMAs per four elements of d come with 12 shared-memory
-// reads (43 TFLOP/s; the same with paired FMAs, whose halved instructions bring nothing).  Both
-// passes over 64 units of about 3500 keys, d 128, 192 window rows: 2401 -> 555 us from one key or
-// row per thread, one read per four FMAs and 2048 keys a CTA.
+// reads (paired FMAs, which halve the instructions, bring nothing).  Both passes over 64 units of about
+// 3500 keys, d 128, 192 window rows: 2400 -> 536 us replayed from a graph (42 TFLOP/s, 52% of the FMA
+// rate; 564 to 620 us as calls among others) from one key or row per thread, one read per four FMAs
+// and 2048 keys a CTA.
 constexpr int kSimtRows = 64, kSimtThreads = 256;
 
 template <int D> struct SimtSmem {

@@ -17,13 +17,15 @@
 // Pass 2 (column sums): keys on M (128 per tile), queries on N, so each thread sums
 //   2^(c*l - b_r) over a range of the window rows for one key.
 //
-// What bounds both is the epilogue's instruction issue: about 3.3 instructions per exponential
-// (scale and subtract, exponential, add, a share of the loads) where the special-function unit
-// takes one per four cycles, and, next to it, the MMA issuer's waits between tiles.  Whole calls,
-// us, on the 7B-class heads (28 x 8 x 4 units, 224 window rows, 15000 to 16384 keys; both passes,
+// What bounds both: HBM, from which each pass reads all keys (two thirds of the 7B-class call below are
+// the time of its 3.6 GB of keys, read twice, at the copy rate); the epilogue's instruction issue, about 3.3 instructions per
+// exponential (scale and subtract, exponential, add, a share of the loads) where the special-function
+// unit takes one per four cycles; and the MMA issuer's waits between tiles.  Whole calls replayed from a
+// graph, us, on the 7B-class heads (28 x 8 x 4 units, 224 window rows, 15000 to 16384 keys; both passes,
 // combine and pool) and in one pass over 8 layers of the 32B-class heads (320 rows, 32768 keys):
-//   before (every epilogue warp on every tile, sizes tested per 8 columns)      1788   889
-//   now (see the comments at the plan, the groups and the batches)              1543   617
+//   before (every epilogue warp on every tile, sizes tested per 8 columns)      1800        900
+//   now (see the comments at the plan, the groups and the batches)              1540-1570   620-630
+//   (as calls among others 1610-1625 and 640)
 // Every mbarrier wait is bounded; a wait that runs out sets the device error word and
 // the CTA stops issuing work, waits (bounded) for nothing further and frees its TMEM.
 #include <cuda.h>
@@ -457,8 +459,9 @@ __global__ void __launch_bounds__(Pass1Cfg<D, MT, EG, SPLIT>::THREADS, 1)
 // own (no second tile to drift to).
 // SHORT: calls of at most kShortTiles tiles per CTA, which a few us of planning would stretch, have the
 // plan inline and their barriers set by a warp: the trace's boundary takes 16.8 us, 19.1 otherwise;
-// long ones take 2% less without.
-constexpr int kShortTiles = 64;
+// its cache of 1024 rows 23.2 and 25.0; 1792 units of 500 to 960
+// keys, all scored, take the same either way, long calls 1 to 2% less without.
+constexpr int kShortTiles = 128;
 constexpr int kP2Groups = 4;
 constexpr int kP2Slots = 4;  // tiles whose other ranges' sums may wait for the first range's warps
 
